@@ -139,25 +139,25 @@ typedef struct {
                           working row of n entries does not fit the walker CTA's shared memory
                           (and n <= 65535), else the dense row; 1 = always the dense row; 2 =
                           always the hash map where it fits (0) */
-  int trisolve_warp_rows; /* level-synchronous triangular solves: a level of at most this many
+  int trisolve_warp_rows; /* level-by-level triangular solves from the chunk streams: a level of at most this many
                           rows, <= 32, is solved by one warp alone, with no barrier among the
                           solving warps after it (the other warps meet it before the next larger
                           level); 0 = every level by all solving warps (0) */
-  int trisolve_group;  /* grouped triangular solves (a partitioned inverse of each factor): at
-                          every factorisation, consecutive levels are merged into groups of at
-                          most this many levels and each row of a group is expanded, by
-                          substitution of the group's earlier rows, into a row that reads only
-                          the input vector and the solution of earlier groups; the solve then
-                          synchronises once per group instead of once per level.  The same
-                          operator as level-by-level substitution in exact arithmetic.  A level
-                          whose expanded rows would exceed the expanded-row capacity
-                          (trisolve_row_cap) starts a new group.  0 or 1: level by level;
-                          ignored with trisolve = 1 (8) */
-  int trisolve_row_cap; /* expanded-row capacity of the grouped solves, in entries: 0 = max(c + 4,
-                          min(2 c, 160)) with c the factor-row capacity; otherwise max(c + 4,
-                          this), at most 480 (0) */
-  int trisolve_lane_entries; /* triangular solves: each row is summed by a group of lanes sized
-                          for at most this many entries a lane on the level's (group's)
+  int trisolve_group;  /* blocked triangular solves (a partitioned inverse of each factor): at
+                          every factorisation the factor's rows are taken in blocks of 8 x this
+                          many (16 x from n = 2048 on; at most 128, and at most the scratch of
+                          trisolve_row_cap) and the diagonal blocks inverted; a block is then
+                          solved in two steps of independent rows, the entries outside the
+                          diagonal block and the inverse, with a synchronisation after each.
+                          The same operator as row-by-row substitution in exact arithmetic.
+                          0 or 1: level by level; ignored with trisolve = 1 (8) */
+  int trisolve_row_cap; /* scratch of the blocked solves, entries a row, which bounds the rows of
+                          a block: 0 = max(c + 4, min(2 c, 160)) with c the factor-row capacity;
+                          otherwise max(c + 4, this), at most 480 (0) */
+  int trisolve_lane_entries; /* triangular solves from the chunk streams (trisolve = 1,
+                          trisolve_warp_rows > 0, or a solve vector that does not fit shared
+                          memory): each row is summed by a group of lanes sized
+                          for at most this many entries a lane on the level's
                           longest row, <= 64; 0 = 2 in FP32, 8 in FP64 (0) */
 } vmc_solver_params;
 
@@ -191,7 +191,8 @@ typedef struct {
                                 matrix/factor values and indices, the vectors read and written */
   int64_t ilu_rows, ilu_elims, ilu_cand; /* ILUTP rows factored, eliminations performed, and
                                 working-row entries before dropping (summed over rows) */
-  int chunks_L, chunks_U;    /* stream chunks of the triangular solves (>= levels)         */
+  int chunks_L, chunks_U;    /* steps of the triangular solves (chunks where they read the
+                                chunk streams)                                               */
   int64_t refactors_async;   /* factorisations adopted from the background factor CTA      */
   int64_t async_wait_cycles; /* solver cycles spent waiting for / adopting them            */
   int64_t async_factor_cycles; /* factor-CTA cycles spent factoring (off the solver's path) */
@@ -199,16 +200,16 @@ typedef struct {
   int async_lag;             /* the refactor_lag in effect (0: in-line refactorisation)     */
   int max_updates;           /* the max_updates in effect                                   */
   int groups_L, groups_U;    /* synchronisation steps of the triangular solves at the last
-                                factorisation (groups of levels; = the level counts when the
-                                solves are not grouped)                                       */
+                                factorisation (two a block at most; = the level counts when the
+                                solves go level by level)                                     */
   int64_t trigger_iterations; /* GMRES iterations until the residual reached trigger_rtol, summed
                                 over solves (the paper's iteration count k1 at its tolerance 1e-6) */
   int64_t reorders_skipped;  /* triggers (monitor, non-convergence, slow) that fired while the
                                 factors were those of a reorder + refactorisation of the very
                                 same matrix (no move accepted since): refactoring it again
                                 would reproduce them, so the solve only restarts           */
-  int64_t stream_bytes;      /* bytes of the L and U chunk streams at the last factorisation:
-                                what one preconditioner apply reads (grouped rows expanded)  */
+  int64_t stream_bytes;      /* bytes of the L and U streams that one preconditioner apply
+                                reads, at the last factorisation                             */
 } vmc_stats;
 
 /* Fill p (host) with the defaults above; VMC_ERR_INVALID for NULL. */

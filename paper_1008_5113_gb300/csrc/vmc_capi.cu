@@ -33,6 +33,15 @@ bool rows_fit_slot(int cap, int lfil_extra, int row_cap) {
   return chunk_bytes(1, 1, mx, 8, true) <= kSlotBytes && chunk_bytes_grouped(1, 1, mx, 8) <= kSlotBytes;
 }
 
+size_t stream_bytes(int n, int capLU, int exmax) {
+  return ((size_t)n * (256 + 12 * (size_t)std::max(capLU, exmax)) + 255) & ~(size_t)255;
+}
+
+int solve_area(int n, int tri_group, size_t tsz) {
+  const size_t extra = tri_group > 1 ? std::min(16 * tri_group, kMaxBlk) : 0;
+  return (int)((((size_t)n + extra) * tsz + 127) / 128 * 128);
+}
+
 void plan_smem(int ybytes, int budget, Params& P, bool allow_sf) {
   int avail = budget;
   P.tri_sf = 0;
@@ -450,12 +459,12 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     o.push_back(cv.take<int>(n));                      // 9 a_len
     o.push_back(cv.take<int>((size_t)n * capLU));      // 10 l_col
     o.push_back(cv.take<double>((size_t)n * capLU));   // 11 l_val64
-    const size_t sbytes = (size_t)n * (256 + 12 * (size_t)std::max(capLU, exmax));
-    o.push_back(cv.take<unsigned char>(sbytes));       // 12 lstream
+    const size_t sbytes = stream_bytes(n, capLU, exmax);
+    o.push_back(cv.take<unsigned char>(2 * sbytes));   // 12 lstream | ustream
     o.push_back(cv.take<int>(n));                      // 13 l_len
     o.push_back(cv.take<int>((size_t)n * capLU));      // 14 u_col
     o.push_back(cv.take<double>((size_t)n * capLU));   // 15 u_val64
-    o.push_back(cv.take<unsigned char>(sbytes));       // 16 ustream
+    o.push_back(0);                                    // 16 (with 12)
     o.push_back(cv.take<int>(n));                      // 17 u_len
     o.push_back(cv.take<double>(n));                   // 18 u_dinv64
     o.push_back(cv.take<int2>(2 * (size_t)n + 2));     // 19 lchunk | uchunk
@@ -493,11 +502,11 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
       // second factor set (same order as offsets 10-30, 47-49), then the snapshot of A
       o.push_back(cv.take<int>((size_t)n * capLU));    // 50 l_col
       o.push_back(cv.take<double>((size_t)n * capLU)); // 51 l_val64
-      o.push_back(cv.take<unsigned char>(sbytes));     // 52 lstream
+      o.push_back(cv.take<unsigned char>(2 * sbytes)); // 52 lstream | ustream
       o.push_back(cv.take<int>(n));                    // 53 l_len
       o.push_back(cv.take<int>((size_t)n * capLU));    // 54 u_col
       o.push_back(cv.take<double>((size_t)n * capLU)); // 55 u_val64
-      o.push_back(cv.take<unsigned char>(sbytes));     // 56 ustream
+      o.push_back(0);                                  // 56 (with 52)
       o.push_back(cv.take<int>(n));                    // 57 u_len
       o.push_back(cv.take<double>(n));                 // 58 u_dinv64
       o.push_back(cv.take<int2>(2 * (size_t)n + 2));   // 59 lchunk | uchunk
@@ -526,11 +535,10 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     }
     o.push_back(cv.take<double2>(n));                  // u_head of factor set 0 (then of set 1)
     if (ctx->pair) o.push_back(cv.take<double2>(n));
-    for (int sset = 0; sset < (ctx->pair ? 2 : 1); ++sset) {  // expanded rows of each factor set
+    for (int sset = 0; sset < (ctx->pair ? 2 : 1); ++sset) {  // inverses of the diagonal blocks of each factor set
       o.push_back(cv.take<int>(n));                      // ex_len
       o.push_back(cv.take<int>((size_t)n * exmax));      // ex_col
       o.push_back(cv.take<double>((size_t)n * exmax));   // ex_val
-      o.push_back(cv.take<int>(n + 1));                  // gptr
     }
     Walker& W = ctx->hw[w];
     std::memset(&W, 0, sizeof(W));
@@ -556,10 +564,10 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
       *out = ctx;
       return fail(ctx, VMC_ERR_CUDA, "no usable CUDA device (shared-memory attributes unavailable)");
     }
-    // grouped solves keep two vectors in shared memory; when two do not fit, one (the
-    // level-by-level solve in place) -- walkers whose two vectors fit it still group
-    const int ybytes1 = (int)(((size_t)ctx->max_n * Tsz + 127) / 128 * 128);
-    const int ybytes = ctx->P.tri_group > 1 ? (int)(((size_t)2 * ctx->max_n * Tsz + 127) / 128 * 128) : ybytes1;
+    // blocked solves keep the solve vector and one block's intermediate vector in shared
+    // memory; when they do not fit, the solve vector alone (the level-by-level solve)
+    const int ybytes1 = solve_area(ctx->max_n, 1, Tsz);
+    const int ybytes = solve_area(ctx->max_n, ctx->P.tri_group, Tsz);
     const int budget1 = optin - stat;
     const int budget2 = per_sm / 2 - 1024 - stat;
     int budget = budget1;
@@ -604,7 +612,8 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     W.l_len = (int*)(A + o[13]);
     W.u_col = (int*)(A + o[14]);
     W.u_val64 = (double*)(A + o[15]);
-    W.ustream = (unsigned char*)(A + o[16]);
+    W.sbytes = stream_bytes(W.n, W.capLU, expanded_row_cap(W.capLU, ctx->row_cap));
+    W.ustream = W.lstream + W.sbytes;
     W.u_len = (int*)(A + o[17]);
     W.u_dinv64 = (double*)(A + o[18]);
     W.lchunk = (int2*)(A + o[19]);
@@ -646,7 +655,6 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
       W.ex_len = (int*)(A + o[e0]);
       W.ex_col = (int*)(A + o[e0 + 1]);
       W.ex_val = (double*)(A + o[e0 + 2]);
-      W.gptr = (int*)(A + o[e0 + 3]);
     }
     W.ctl = ctx->dCtl + w;
     const Layout& L = lay[w];
@@ -675,7 +683,7 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
       W1.l_len = (int*)(A + o[53]);
       W1.u_col = (int*)(A + o[54]);
       W1.u_val64 = (double*)(A + o[55]);
-      W1.ustream = (unsigned char*)(A + o[56]);
+      W1.ustream = W1.lstream + W1.sbytes;
       W1.u_len = (int*)(A + o[57]);
       W1.u_dinv64 = (double*)(A + o[58]);
       W1.lchunk = (int2*)(A + o[59]);
@@ -695,10 +703,9 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
       W1.lvl_nchunk = (int*)(A + o[72]);
       W1.seg_meta = (int4*)(A + o[73]);
       W1.u_head = (double2*)(A + o[83]);
-      W1.ex_len = (int*)(A + o[88]);
-      W1.ex_col = (int*)(A + o[89]);
-      W1.ex_val = (double*)(A + o[90]);
-      W1.gptr = (int*)(A + o[91]);
+      W1.ex_len = (int*)(A + o[87]);
+      W1.ex_col = (int*)(A + o[88]);
+      W1.ex_val = (double*)(A + o[89]);
       W0.snap_len = (int*)(A + o[74]);
       W0.snap_col = (int*)(A + o[75]);
       W0.snap_val = (double*)(A + o[76]);

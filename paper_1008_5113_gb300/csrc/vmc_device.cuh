@@ -35,6 +35,7 @@ constexpr int kSlotBytes = 8192;  // smallest ring slot (a slot holds the larges
 constexpr int kMaxSlots = 8;      // ring depth (chunks in flight)
 constexpr int kChunkHdr = 80;     // chunk header bytes: int4 + 8 next-chunk descriptors
 constexpr int kMaxSeg = 32;       // levels (segments) per chunk at most
+constexpr int kMaxBlk = 128;      // blocked solves: rows of a block at most
 // phase indices of Ctl::cyc
 enum : int { PH_BUILD = 0, PH_FIRST = 1, PH_REFINE = 2, PH_FACTOR = 3, PH_REORDER = 4, PH_COMMIT = 5, PH_STEP = 6,
              PH_TRI = 7, PH_CHAIN = 8, PH_SPMV = 9, PH_ORTH = 10, PH_RESID = 11, PH_ILUTP = 12, PH_LEVELS = 13, PH_TRIWAIT = 14,
@@ -56,7 +57,8 @@ struct Ctl {
   int last_pivots;
   int last_breakdown;
   int nchunk_l, nchunk_u;
-  int ngrp_l, ngrp_u;  // barriers of the triangular solves (groups; = levels when not grouped)
+  int ngrp_l, ngrp_u;  // barriers of the triangular solves (steps; = levels when level by level)
+  int tri_tasks;       // 1: the streams in use are task streams (vmc_blocks.cuh)
   long long stream_bytes;  // bytes of the L and U chunk streams (read by every preconditioner apply)
   double pend_r[3];
   double pend_ratio;
@@ -114,10 +116,13 @@ struct Walker {
   int* u_col; double* u_val64; int* u_len;
   double* u_dinv64;
   double2* u_head;        // per U row {1 / u_rr, length}, written by the shared-memory ILUTP
-  // grouped triangular solves: expanded rows (exmax entries each) and group row pointers
-  int exmax; int* ex_len; int* ex_col; double* ex_val; int* gptr;
-  // level-ordered chunk streams of L and U for the staged triangular solves
+  // blocked triangular solves: scratch of exmax entries a row for the inverses of the
+  // diagonal blocks
+  int exmax; int* ex_len; int* ex_col; double* ex_val;
+  // level-ordered chunk streams of L and U for the staged triangular solves, or the block
+  // streams of both from lstream on (ustream = lstream + sbytes)
   unsigned char* lstream; unsigned char* ustream;
+  size_t sbytes;
   int2* lchunk; int2* uchunk;   // per chunk {byte offset, bytes}
   int4* chunk_meta;             // scratch per chunk {first segment, segments, rows, entries}
   int4* seg_meta;               // scratch per segment {first row in level order, rows, entries, 0}
@@ -169,7 +174,7 @@ struct Params {
   int trig_its;     // ... within this many GMRES iterations (all cycles)
   int ilu_variant;  // 0: auto (hash working row where the dense one misses shared memory); 1: dense; 2: hash
   int warp_rows;    // levels of at most this many rows: triangular-solve rows by one warp, no barrier
-  int tri_group;    // > 1: grouped triangular solves, at most this many levels per group
+  int tri_group;    // > 1: blocked triangular solves, blocks of 8 x this many rows
   int lane_entries; // entries per lane the triangular solves' lane groups are sized for
   // budgeted advance of the persistent engine: the walkers claim moves one at a time from
   // *budget_ctr until budget_total are claimed (nullptr: fixed sweeps)
@@ -211,21 +216,30 @@ struct __align__(16) Shared {
   double dflag[8];
 };
 
-// Grouped triangular solves (expand_groups): on when asked for, the walker has the
-// scratch for the expanded rows, its two solve vectors fit the shared-memory solve area,
-// and one hash accumulator per warp of the CTA fits the dynamic shared memory (else the
-// level-by-level solve, in place on one vector).  Decided the same way at factorisation
-// and solve.
-__device__ __forceinline__ int group_hash_slots(int exmax) {
-  int hs = 64;
-  while (hs < 2 * exmax) hs <<= 1;
-  return hs;
+// Blocked triangular solves (vmc_blocks.cuh): rows of a block.  From n = 2048 on the inverses
+// of 128-row blocks stay sparse (n = 4096, fill limit 32: 2.18 MB of streams against 2.23 MB
+// with 64 rows) and half the steps win: 80 against 98 us for L and U in FP32; below, the
+// larger blocks' inverses fill in (n = 343: 286 against 234 KB, 10.7 against 10.3 us).
+__device__ __forceinline__ int block_rows(const Walker& w, const Params& P) {
+  return min(min((w.n >= 2048 ? 16 : 8) * P.tri_group, kMaxBlk), w.exmax);
 }
+constexpr int kLaneEntries = 8;  // entries of a lane in one task of a warp
+// Bytes of a task: words, sources, values.
+__host__ __device__ __forceinline__ constexpr int task_bytes(int tsz) { return 128 + 512 + 32 * kLaneEntries * tsz; }
+// Tasks of every warp that the shared memory after the solve area holds.
 template <typename T>
-__device__ __forceinline__ bool grouped_solves(const Walker& w, const Params& P) {
-  return P.tri_group > 1 && w.ex_col != nullptr && P.y_smem &&
-         2 * (size_t)w.n * sizeof(T) <= (size_t)P.y_bytes &&  // both solve vectors in shared memory
-         (size_t)(blockDim.x >> 5) * 12u * (size_t)group_hash_slots(w.exmax) <= (size_t)P.dsm_bytes;
+__device__ __forceinline__ int tasks_ahead(const Params& P) {
+  return P.ring_slots * P.slot_bytes / ((int)(blockDim.x >> 5) * task_bytes((int)sizeof(T)));
+}
+// Task streams serve the solves when the solve vector (and one block's intermediate one)
+// fit the shared-memory solve area, with 16-bit indices, blocks of a useful size and two
+// tasks a warp; else (and for the synchronisation-free solves and trisolve_warp_rows) the
+// level-ordered chunk streams.
+template <typename T>
+__device__ __forceinline__ bool task_solves(const Walker& w, const Params& P) {
+  const int B = P.tri_group > 1 ? block_rows(w, P) : 0;
+  return P.y_smem && !P.tri_sf && P.warp_rows == 0 && (P.tri_group <= 1 || (w.ex_col != nullptr && B >= 16)) &&
+         w.n + B < 0xffff && (size_t)(w.n + B) * sizeof(T) <= (size_t)P.y_bytes && tasks_ahead<T>(P) >= 2;
 }
 
 // ---- block-wide copies with several loads in flight per thread ---------------

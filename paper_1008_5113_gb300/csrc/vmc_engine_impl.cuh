@@ -285,6 +285,7 @@ __device__ void af_swap(const Walker& w0, const Params& P, Shared& sh) {
     c->ngrp_l = sc->ngrp_l; c->ngrp_u = sc->ngrp_u;
     c->nchunk_l = sc->nchunk_l; c->nchunk_u = sc->nchunk_u;
     c->stream_bytes = sc->stream_bytes;
+    c->tri_tasks = sc->tri_tasks;
     c->nnz_LU = sc->nnz_LU; c->nnz_A = sc->nnz_A;
     c->p_lfil = sc->p_lfil; c->last_pivots = sc->last_pivots; c->last_breakdown = 0;
     c->active = c->af_target;

@@ -88,6 +88,10 @@ cudaError_t launch_bench_T(const LaunchCfg& L, const Walker* W, int nwalk, const
 void plan_smem(int ybytes, int budget, Params& P, bool allow_sf);
 // Entries of an expanded row of the grouped triangular solves (a multiple of 4).
 int expanded_row_cap(int capLU, int row_cap);
+// Bytes of one factor's stream buffer; a factor set has two side by side.
+size_t stream_bytes(int n, int capLU, int exmax);
+// Bytes of the shared-memory solve area for systems of up to n particles.
+int solve_area(int n, int tri_group, size_t tsz);
 bool rows_fit_slot(int cap, int lfil_extra, int row_cap);
 
 // host-side geometry and layout

@@ -135,32 +135,6 @@ __device__ __forceinline__ void ring_init(Shared& sh, const Params& P) {
   __syncthreads();
 }
 
-// Entries of a grouped chunk (the layout of chunk_bytes_grouped): entry t is (column
-// offset, value).
-template <typename T>
-struct GroupedEntries;
-template <>
-struct GroupedEntries<float> {
-  const float2* p;
-  __device__ __forceinline__ GroupedEntries(const unsigned char* ent, int) : p((const float2*)ent) {}
-  __device__ __forceinline__ void get(int t, int& c, float& v) const {
-    const float2 e = p[t];
-    c = __float_as_int(e.x);
-    v = e.y;
-  }
-};
-template <>
-struct GroupedEntries<double> {
-  const int* c;
-  const double* v;
-  __device__ __forceinline__ GroupedEntries(const unsigned char* ent, int ne)
-      : c((const int*)ent), v((const double*)(ent + pad16(4 * ne))) {}
-  __device__ __forceinline__ void get(int t, int& cc, double& vv) const {
-    cc = c[t];
-    vv = v[t];
-  }
-};
-
 // Producer of the chunk streams (lane 0 of the last warp): streams the factor's chunks
 // into the ring with bulk copies, refilling a slot once the consumers have released it
 // (the slot's "empty" barrier).  Returns the cycles spent waiting for free slots.
@@ -232,80 +206,6 @@ __device__ __forceinline__ void tri_staged(const Walker& w, const Params& P, boo
       const int* cl = st + pad4(nr + 1);
       const T* vl = (const T*)(cl + pad4(ne));
       const T* dv = (const T*)((const unsigned char*)vl + pad16((int)sizeof(T) * ne));
-      if (hd.w) {
-        // grouped form: the rows of a segment (group) are independent; each is a dot
-        // product with the solution and input vectors at offsets from y (row descriptor
-        // {output, first, end}; entries as (column, value) pairs)
-        const int4* desc = (const int4*)(ch + kChunkHdr + 16 * nseg);
-        const GroupedEntries<T> ent(ch + kChunkHdr + 16 * nseg + 16 * nr, ne);
-        for (int sgi = 0; sgi < nseg; ++sgi) {
-          const int4 sm = seg[sgi];
-          const int r0 = sm.x, sr = sm.y, gs = sm.z;
-          const int G = 1 << gs;
-          const int gl = tid & (G - 1);
-          const int ng = nct >> gs;
-          for (int base = 0; base < sr; base += ng) {  // same trip count in every lane
-            const int i = r0 + base + (tid >> gs);
-            const bool on = base + (tid >> gs) < sr;
-            T part = 0;
-            int r = 0;
-            if (on) {
-              // expanded rows are long (up to exmax entries): FP32 keeps four entries in
-              // flight per lane; FP64 two (every extra partial sum costs an FP64 add)
-              const int4 d = desc[i];
-              r = d.x;
-              const int e = d.z;
-              int t = d.y + gl;
-              if constexpr (sizeof(T) == 4) {
-                T p1 = 0, p2 = 0, p3 = 0;
-                for (; t + 3 * G < e; t += 4 * G) {
-                  int c0, c1, c2, c3;
-                  T v0, v1, v2, v3;
-                  ent.get(t, c0, v0);
-                  ent.get(t + G, c1, v1);
-                  ent.get(t + 2 * G, c2, v2);
-                  ent.get(t + 3 * G, c3, v3);
-                  part += v0 * y[c0];
-                  p1 += v1 * y[c1];
-                  p2 += v2 * y[c2];
-                  p3 += v3 * y[c3];
-                }
-                for (; t < e; t += G) {
-                  int c0;
-                  T v0;
-                  ent.get(t, c0, v0);
-                  part += v0 * y[c0];
-                }
-                part = (part + p1) + (p2 + p3);
-              } else {
-                T p1 = 0;
-                for (; t + G < e; t += 2 * G) {
-                  int c0, c1;
-                  T v0, v1;
-                  ent.get(t, c0, v0);
-                  ent.get(t + G, c1, v1);
-                  part += v0 * y[c0];
-                  p1 += v1 * y[c1];
-                }
-                if (t < e) {
-                  int c0;
-                  T v0;
-                  ent.get(t, c0, v0);
-                  part += v0 * y[c0];
-                }
-                part += p1;
-              }
-            }
-            for (int o = G >> 1; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o, G);
-            if (on && gl == 0) y[r] = part;
-          }
-          asm volatile("bar.sync 1, %0;" ::"r"(nct) : "memory");  // group barrier (consumers)
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.ebar[slot]);
-        if (++slot == S) { slot = 0; parity ^= 1u; }
-        continue;
-      }
       for (int sgi = 0; sgi < nseg; ++sgi) {
         const int4 sm = seg[sgi];
         const int r0 = sm.x, sr = sm.y;
@@ -505,18 +405,8 @@ __device__ __forceinline__ void tri_syncfree(const Walker& w, const Params& P, b
 template <typename T>
 __device__ __forceinline__ const T* tri_both(const Walker& w, const Params& P, const T* v, Shared& sh) {
   const int n = w.n, tid = threadIdx.x, nt = blockDim.x;
+  if (w.ctl->tri_tasks) return tri_tasks<T>(w, P, v);
   T* y = P.y_smem ? (T*)dyn_smem() : (T*)w.tv;
-  if (grouped_solves<T>(w, P)) {
-    // two vectors [a | b]: v goes to b; L writes y_L into a reading b at offset +n; U
-    // writes x into b (v is no longer needed) reading y_L at offset -n
-    T* a = y;
-    T* b = y + n;
-    block_copy(b, v, n);
-    __syncthreads();
-    tri_staged<T>(w, P, false, a, sh);
-    tri_staged<T>(w, P, true, b, sh);
-    return b;
-  }
   if (P.tri_sf) {
     T* x2 = (T*)(dyn_smem() + P.y_half);
     for (int i = tid; i < n; i += nt) { y[i] = Pending<T>::value(); x2[i] = Pending<T>::value(); }

@@ -136,7 +136,7 @@ extern "C" vmc_status vmc_ratio_noalloc(const vmc_system* sys, const vmc_solver_
   const int pmax = p.lfil_extra >= 0 ? p.lfil_extra : (cap + 1) / 2;
   const int capLU = (cap + pmax + 2 + 3) / 4 * 4;
   const int exmax = expanded_row_cap(capLU, p.trisolve_row_cap);
-  const size_t sbytes = (size_t)n * (256 + 12 * (size_t)std::max(capLU, exmax));
+  const size_t sbytes = stream_bytes(n, capLU, exmax);
 
   // carve the walker workspace out of the scratch array
   Off o;
@@ -145,9 +145,9 @@ extern "C" vmc_status vmc_ratio_noalloc(const vmc_system* sys, const vmc_solver_
   const size_t oAc = o.take<int>((size_t)n * cap), oAv = o.take<double>((size_t)n * cap);
   const size_t oAv32 = o.take<float>((size_t)n * cap), oAl = o.take<int>(n);
   const size_t oLc = o.take<int>((size_t)n * capLU), oLv = o.take<double>((size_t)n * capLU);
-  const size_t oLs = o.take<unsigned char>(sbytes), oLl = o.take<int>(n);
+  const size_t oLs = o.take<unsigned char>(2 * sbytes), oLl = o.take<int>(n);
   const size_t oUc = o.take<int>((size_t)n * capLU), oUv = o.take<double>((size_t)n * capLU);
-  const size_t oUs = o.take<unsigned char>(sbytes), oUl = o.take<int>(n), oUd = o.take<double>(n);
+  const size_t oUl = o.take<int>(n), oUd = o.take<double>(n);
   const size_t oCh = o.take<int2>(2 * (size_t)n + 2);
   const size_t oPm = o.take<int>(n), oIp = o.take<int>(n), oLvl = o.take<int>(n), oUvl = o.take<int>(n);
   const size_t oLlp = o.take<int>(n + 1), oLlr = o.take<int>(n), oUlp = o.take<int>(n + 1), oUlr = o.take<int>(n);
@@ -163,7 +163,6 @@ extern "C" vmc_status vmc_ratio_noalloc(const vmc_system* sys, const vmc_solver_
   const size_t oSeg = o.take<int4>(2 * (size_t)n + 2);
   const size_t oUh = o.take<double2>(n);
   const size_t oExl = o.take<int>(n), oExc = o.take<int>((size_t)n * exmax), oExv = o.take<double>((size_t)n * exmax);
-  const size_t oGp = o.take<int>(n + 1);
   const size_t oCtl = o.take<Ctl>(1), oW = o.take<Walker>(1);
   const size_t used = o.off;
   if (used > kNoAllocBytes)
@@ -184,12 +183,11 @@ extern "C" vmc_status vmc_ratio_noalloc(const vmc_system* sys, const vmc_solver_
   W.a_col = (int*)(base + oAc); W.a_val = (double*)(base + oAv); W.a_val32 = (float*)(base + oAv32);
   W.a_len = (int*)(base + oAl);
   W.l_col = (int*)(base + oLc); W.l_val64 = (double*)(base + oLv); W.lstream = base + oLs; W.l_len = (int*)(base + oLl);
-  W.u_col = (int*)(base + oUc); W.u_val64 = (double*)(base + oUv); W.ustream = base + oUs; W.u_len = (int*)(base + oUl);
+  W.u_col = (int*)(base + oUc); W.u_val64 = (double*)(base + oUv); W.sbytes = sbytes; W.ustream = W.lstream + sbytes; W.u_len = (int*)(base + oUl);
   W.u_dinv64 = (double*)(base + oUd);
   W.u_head = (double2*)(base + oUh);
   W.exmax = exmax;
   W.ex_len = (int*)(base + oExl); W.ex_col = (int*)(base + oExc); W.ex_val = (double*)(base + oExv);
-  W.gptr = (int*)(base + oGp);
   W.lchunk = (int2*)(base + oCh); W.uchunk = W.lchunk + (n + 1);
   W.perm = (int*)(base + oPm); W.iperm = (int*)(base + oIp); W.lev_l = (int*)(base + oLvl); W.lev_u = (int*)(base + oUvl);
   W.l_lvl_ptr = (int*)(base + oLlp); W.l_lvl_rows = (int*)(base + oLlr);
@@ -226,8 +224,8 @@ extern "C" vmc_status vmc_ratio_noalloc(const vmc_system* sys, const vmc_solver_
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const int stat = kernel_static_smem(fp64);
   if (optin <= 0 || stat <= 0) return fail(VMC_ERR_CUDA, "no usable CUDA device");
-  const int ybytes1 = (int)(((size_t)n * Tsz + 127) / 128 * 128);
-  const int ybytes = P.tri_group > 1 ? (int)(((size_t)2 * n * Tsz + 127) / 128 * 128) : ybytes1;
+  const int ybytes1 = solve_area(n, 1, Tsz);
+  const int ybytes = solve_area(n, P.tri_group, Tsz);
   const int budget = optin - stat;
   plan_smem(ybytes, budget, P, p.trisolve == 1);
   if (!P.y_smem && ybytes != ybytes1) plan_smem(ybytes1, budget, P, p.trisolve == 1);

@@ -7,6 +7,7 @@
 //     Eq. 14: A Q ~ L U);
 //   * level sets of L and U for the parallel triangular solves.
 #pragma once
+#include "vmc_blocks.cuh"
 #include "vmc_geom.cuh"
 
 namespace vmc {
@@ -911,24 +912,18 @@ __device__ __noinline__ int ilutp_warp_hash(const Walker& w, const Params& P, Sh
 // chunks.  Block-wide (packing by thread 0: sequential over levels, and over rows
 // only inside levels that must be split).
 // ---------------------------------------------------------------------------
-// Grouped form (expanded = true): the segments are groups of consecutive levels and the
-// rows are the expanded rows of expand_groups (no diagonal array; chunk header .w = 1).
 template <typename T>
-__device__ int build_stream(const Walker& w, const Params& P, bool upper, int nlev, Shared& sh,
-                            bool expanded = false) {
+__device__ int build_stream(const Walker& w, const Params& P, bool upper, int nlev, Shared& sh) {
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
-  const int* lptr = expanded ? w.gptr : (upper ? w.u_lvl_ptr : w.l_lvl_ptr);
+  const int* lptr = upper ? w.u_lvl_ptr : w.l_lvl_ptr;
   const int* rows = upper ? w.u_lvl_rows : w.l_lvl_rows;
-  const int* len = expanded ? w.ex_len : (upper ? w.u_len : w.l_len);
-  const int* colv = expanded ? w.ex_col : (upper ? w.u_col : w.l_col);
-  const double* valv = expanded ? w.ex_val : (upper ? w.u_val64 : w.l_val64);
+  const int* len = upper ? w.u_len : w.l_len;
+  const int* colv = upper ? w.u_col : w.l_col;
+  const double* valv = upper ? w.u_val64 : w.l_val64;
   int2* tab = upper ? w.uchunk : w.lchunk;
   unsigned char* stream = upper ? w.ustream : w.lstream;
-  const int tsz = (int)sizeof(T), capLU = expanded ? w.exmax : w.capLU;
-  const bool with_dv = upper && !expanded;
-  auto cbytes = [&](int ns, int r, int e) {
-    return expanded ? chunk_bytes_grouped(ns, r, e, tsz) : chunk_bytes(ns, r, e, tsz, with_dv);
-  };
+  const int tsz = (int)sizeof(T), capLU = w.capLU;
+  auto cbytes = [&](int ns, int r, int e) { return chunk_bytes(ns, r, e, tsz, upper); };
   const int SB = P.slot_bytes;
   const int nct = nt - 32;  // consumer threads of the solve
   // entries per level and the level's lane-group size (warp per level).  The group size
@@ -969,7 +964,7 @@ __device__ int build_stream(const Walker& w, const Params& P, bool upper, int nl
       const int gsl = w.lvl_nchunk[lev] >> 28;
       int gw = gsl;
       while (gw > 0 && (lr << gw) > 32) --gw;
-      const int wmode = (!expanded && lr <= P.warp_rows && (lr << gw) <= 32) ? gw + 1 : 0;
+      const int wmode = (lr <= P.warp_rows && (lr << gw) <= 32) ? gw + 1 : 0;
       const int lgs = gsl | (wmode << 8);
       if (cs < kMaxSeg && cbytes(cs + 1, cr + lr, ce + le) <= SB) {
         w.seg_meta[nseg++] = make_int4(q, lr, le, lgs);  // the whole level joins the open chunk
@@ -1013,56 +1008,6 @@ __device__ int build_stream(const Walker& w, const Params& P, bool upper, int nl
   for (int c = tid; c < nch_total; c += nt) tab[c].x = w.lvl_cur[c];
   __syncthreads();
   // fill the chunks, one warp per chunk
-  if (expanded) {
-    for (int c = wid; c < nch_total; c += nw) {
-      const int4 cm = w.chunk_meta[c];
-      const int seg0 = cm.x, nseg = cm.y, nr = cm.z, ne = cm.w;
-      unsigned char* base = stream + tab[c].x;
-      int4* seg = (int4*)(base + kChunkHdr);
-      int4* desc = (int4*)(base + kChunkHdr + 16 * nseg);
-      unsigned char* ent = base + kChunkHdr + 16 * nseg + 16 * nr;
-      if (lane == 0) *(int4*)base = make_int4(nseg, nr, ne, 1);
-      if (lane < kMaxSlots)
-        ((int2*)(base + 16))[lane] = c + 1 + lane < nch_total ? tab[c + 1 + lane] : make_int2(0, 0);
-      int rbase = 0, carry = 0;
-      for (int sgi = 0; sgi < nseg; ++sgi) {
-        const int4 sm = w.seg_meta[seg0 + sgi];
-        const int q0 = sm.x, sr = sm.y;
-        if (lane == 0) seg[sgi] = make_int4(rbase, sr, sm.w & 0xff, 0);
-        for (int b0 = 0; b0 < sr; b0 += 32) {
-          const int i = b0 + lane;
-          const int r = i < sr ? rows[q0 + i] : 0;
-          const int L = i < sr ? len[r] : 0;
-          int inc = L;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += v;
-          }
-          if (i < sr) desc[rbase + i] = make_int4(r, carry + inc - L, carry + inc, 0);
-          carry += __shfl_sync(0xffffffffu, inc, 31);
-        }
-        rbase += sr;
-      }
-      __syncwarp();
-      for (int i = 0; i < nr; ++i) {
-        const int4 d = desc[i];
-        const int r = d.x, b = d.y, L = d.z - d.y;
-        for (int t = lane; t < L; t += 32) {
-          const int col = colv[(size_t)r * capLU + t];
-          const double val = valv[(size_t)r * capLU + t];
-          if (tsz == 4) {
-            reinterpret_cast<float2*>(ent)[b + t] = make_float2(__int_as_float(col), (float)val);
-          } else {
-            reinterpret_cast<int*>(ent)[b + t] = col;
-            reinterpret_cast<double*>(ent + pad16(4 * ne))[b + t] = val;
-          }
-        }
-      }
-    }
-    __syncthreads();
-    return nch_total;
-  }
   for (int c = wid; c < nch_total; c += nw) {
     const int4 cm = w.chunk_meta[c];
     const int seg0 = cm.x, nseg = cm.y, nr = cm.z, ne = cm.w;
@@ -1073,7 +1018,7 @@ __device__ int build_stream(const Walker& w, const Params& P, bool upper, int nl
     int* cl = st + pad4(nr + 1);
     T* vl = (T*)(cl + pad4(ne));
     T* dv = (T*)((unsigned char*)vl + pad16(tsz * ne));
-    if (lane == 0) *(int4*)base = make_int4(nseg, nr, ne, expanded ? 1 : 0);
+    if (lane == 0) *(int4*)base = make_int4(nseg, nr, ne, 0);
     if (lane < kMaxSlots) ((int2*)(base + 16))[lane] = c + 1 + lane < nch_total ? tab[c + 1 + lane] : make_int2(0, 0);
     int rbase = 0, carry = 0;
     for (int sgi = 0; sgi < nseg; ++sgi) {
@@ -1093,7 +1038,7 @@ __device__ int build_stream(const Walker& w, const Params& P, bool upper, int nl
         if (i < sr) {
           rws[rbase + i] = r;
           st[rbase + i] = carry + inc - L;
-          if (with_dv) dv[rbase + i] = (T)w.u_dinv64[r];
+          if (upper) dv[rbase + i] = (T)w.u_dinv64[r];
         }
         carry += __shfl_sync(0xffffffffu, inc, 31);
       }
@@ -1114,164 +1059,10 @@ __device__ int build_stream(const Walker& w, const Params& P, bool upper, int nl
   return nch_total;
 }
 
-// ---------------------------------------------------------------------------
-// Grouped triangular solves (a partitioned inverse of the factor).  Consecutive levels
-// of L (of U) are merged into groups of at most P.tri_group levels; every row of a group
-// is expanded by substituting the rows of the same group it depends on, so that it
-// reads only the input vector v and solution entries of earlier groups:
-//   L:  y_r = v_r - sum_c L_rc y_c          ->  y_r = sum_q a_rq v_q + sum_{c earlier} b_rc y_c
-//   U:  x_r = (y_r - sum_c U_rc x_c) / U_rr  ->  x_r = sum_q a_rq y_q + sum_{c earlier} b_rc x_c
-// (q over the row and its ancestors inside the group).  The rows of a group are then
-// independent, and the solve needs one barrier per group instead of one per level.  The
-// operator is the same as the level-by-level substitution in exact arithmetic (the
-// coefficients are formed in FP64 and rounded once to the working precision).  Indices
-// of the expanded rows are offsets from the solution vector: c in [0, n) the solution
-// entry c; the input entry q at n + q for L (the input vector follows the solution) and
-// at q - n for U (it precedes it: the L solution is U's input).  A level joins the open
-// group only while every expanded row of it stays within w.exmax entries; otherwise it
-// starts a new group.
-// Block-wide; one warp per row with a hash accumulator of 2 exmax slots in the dynamic
-// shared memory (idle after the factorisation).  Writes w.gptr (row pointer of each
-// group into the level-ordered rows), w.ex_len/ex_col/ex_val; returns the group count.
-// ---------------------------------------------------------------------------
-template <typename T>
-__device__ __noinline__ int expand_groups(const Walker& w, const Params& P, bool upper, int nlev, Shared& sh) {
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
-  const int n = w.n, capLU = w.capLU, EX = w.exmax;
-  const int* lptr = upper ? w.u_lvl_ptr : w.l_lvl_ptr;
-  const int* rows = upper ? w.u_lvl_rows : w.l_lvl_rows;
-  const int* flen = upper ? w.u_len : w.l_len;
-  const int* fcol = upper ? w.u_col : w.l_col;
-  const double* fval = upper ? w.u_val64 : w.l_val64;
-  const int* lev = upper ? w.lev_u : w.lev_l;
-  const int hs = group_hash_slots(EX);  // per-warp table: at most half full
-  const int hmask = hs - 1;
-  constexpr int kEmpty = (int)0x80000000;  // keys are offsets in [-n, 2n)
-  const int in_off = upper ? -n : n;
-  int* hkey = reinterpret_cast<int*>(dyn_smem()) + (size_t)wid * hs * 3;  // keys, then values (8-byte aligned)
-  double* hval = reinterpret_cast<double*>(hkey + hs + (hs & 1));
-  auto add = [&](int key, double v, int& cnt, bool& over, bool active) {
-    // lanes with active = true add distinct keys; returns the updated count (uniform)
-    bool ins = false;
-    int h = 0;
-    if (active) {
-      h = (int)(((unsigned)key * 0x9E3779B1u) >> 7) & hmask;
-      for (int probe = 0; probe < hs; ++probe) {
-        const int k = hkey[h];
-        if (k == key) { hval[h] += v; break; }
-        if (k == kEmpty) {
-          const int old = atomicCAS(&hkey[h], kEmpty, key);
-          if (old == kEmpty) { hval[h] = v; ins = true; break; }
-          if (old == key) { hval[h] += v; break; }
-        }
-        h = (h + 1) & hmask;
-      }
-    }
-    cnt += __popc(__ballot_sync(0xffffffffu, ins));
-    if (cnt > EX) over = true;
-    __syncwarp();
-  };
-  // expand the rows of level lv with the open group starting at level g; returns true
-  // (block-uniform) when a row exceeded exmax entries
-  auto expand_level = [&](int lv, int g) -> bool {
-    bool any_over = false;
-    for (int q = lptr[lv] + wid; q < lptr[lv + 1]; q += nw) {
-      const int r = rows[q];
-      for (int i = lane; i < hs; i += 32) hkey[i] = kEmpty;
-      __syncwarp();
-      const double d = upper ? w.u_dinv64[r] : 1.0;
-      int cnt = 0;
-      bool over = false;
-      add(in_off + r, d, cnt, over, lane == 0);
-      const int L = flen[r];
-      const int* rc = fcol + (size_t)r * capLU;
-      const double* rv = fval + (size_t)r * capLU;
-      for (int t0 = 0; t0 < L; t0 += 32) {  // dependencies on earlier groups
-        const int t = t0 + lane;
-        const bool act = t < L && lev[rc[t]] < g;
-        add(act ? rc[t] : 0, act ? -d * rv[t] : 0.0, cnt, over, act);
-      }
-      for (int t = 0; t < L && !over; ++t) {  // dependencies inside the group: substitute
-        const int c = rc[t];
-        if (lev[c] < g) continue;
-        const double coef = -d * rv[t];
-        const int el = w.ex_len[c];
-        const int* ec = w.ex_col + (size_t)c * EX;
-        const double* ev = w.ex_val + (size_t)c * EX;
-        for (int e0 = 0; e0 < el; e0 += 32) {
-          const int e = e0 + lane;
-          add(e < el ? ec[e] : 0, e < el ? coef * ev[e] : 0.0, cnt, over, e < el);
-        }
-      }
-      // write the expanded row (slot order)
-      int outc = 0;
-      for (int i0 = 0; i0 < hs; i0 += 32) {
-        const int i = i0 + lane;
-        const bool k = !over && hkey[i] != kEmpty;
-        const unsigned m = __ballot_sync(0xffffffffu, k);
-        const int slot = outc + __popc(m & lanemask_lt());
-        if (k && slot < EX) {
-          w.ex_col[(size_t)r * EX + slot] = hkey[i];
-          w.ex_val[(size_t)r * EX + slot] = hval[i];
-        }
-        outc += __popc(m);
-      }
-      if (lane == 0) w.ex_len[r] = over ? 0 : min(outc, EX);
-      any_over |= over;
-      __syncwarp();
-    }
-    const int o = block_max_int(any_over ? 1 : 0, sh);  // ends synchronised
-    return o != 0;
-  };
-  int g0 = 0, ngrp = 0;
-  if (tid == 0) w.gptr[0] = 0;
-  for (int lv = 0; lv < nlev; ++lv) {
-    const bool join = lv > 0 && lv - g0 < P.tri_group;
-    bool newg = !join;
-    if (join && expand_level(lv, g0)) newg = true;
-    if (newg) {
-      if (lv > 0) {
-        ++ngrp;
-        if (tid == 0) w.gptr[ngrp] = lptr[lv];
-      }
-      g0 = lv;
-      expand_level(lv, lv);
-    }
-  }
-  ++ngrp;
-  if (tid == 0) w.gptr[ngrp] = lptr[nlev];
+// Packs both level sets (counting sort by level).  Block-wide, ends synchronised.
+static __device__ __noinline__ void level_sets(const Walker& w, int nll, int nlu) {
+  const int n = w.n, tid = threadIdx.x, nt = blockDim.x;
   __syncthreads();
-  return ngrp;
-}
-
-// Block-wide: relabel U columns to factor labels, compute U levels (warp 0,
-// reverse order) and pack both level sets (counting sort by level).
-template <typename T>
-__device__ __noinline__ void relabel_and_levels(const Walker& w, const Params& P, Shared& sh) {
-  const int n = w.n, tid = threadIdx.x, nt = blockDim.x, capLU = w.capLU;
-  for (int idx = tid; idx < n * capLU; idx += nt) {
-    const int r = idx / capLU, t = idx - r * capLU;
-    if (t < w.u_len[r]) w.u_col[idx] = w.iperm[w.u_col[idx]];
-  }
-  __syncthreads();
-  if (tid < 32) {
-    const int lane = tid;
-    for (int r = n - 1; r >= 0; --r) {
-      const int ul = w.u_len[r];
-      int lv = -1;
-      for (int t = lane; t < ul; t += 32) lv = max(lv, w.lev_u[w.u_col[(size_t)r * capLU + t]]);
-      lv = warp_max_int(lv);
-      if (lane == 0) w.lev_u[r] = lv + 1;
-      __syncwarp();
-    }
-  }
-  __syncthreads();
-  // level counts
-  int mlv = 0, muv = 0;
-  for (int r = tid; r < n; r += nt) { mlv = max(mlv, w.lev_l[r]); muv = max(muv, w.lev_u[r]); }
-  const int ml = block_max_int(mlv, sh);
-  const int mu = block_max_int(muv, sh);
-  const int nll = ml + 1, nlu = mu + 1;
   for (int q = tid; q <= n; q += nt) { w.l_lvl_ptr[q] = 0; w.u_lvl_ptr[q] = 0; }
   __syncthreads();
   for (int r = tid; r < n; r += nt) {
@@ -1291,25 +1082,88 @@ __device__ __noinline__ void relabel_and_levels(const Walker& w, const Params& P
   for (int q = tid; q < nlu; q += nt) w.lvl_cur[q] = w.u_lvl_ptr[q];
   __syncthreads();
   for (int r = tid; r < n; r += nt) w.u_lvl_rows[atomicAdd(&w.lvl_cur[w.lev_u[r]], 1)] = r;
-  if (tid == 0) { w.ctl->nlev_l = nll; w.ctl->nlev_u = nlu; }
   __syncthreads();
-  int ncl, ncu;
-  if (grouped_solves<T>(w, P)) {
-    const int gl = expand_groups<T>(w, P, false, nll, sh);
-    ncl = build_stream<T>(w, P, false, gl, sh, true);
-    const int gu = expand_groups<T>(w, P, true, nlu, sh);
-    ncu = build_stream<T>(w, P, true, gu, sh, true);
-    if (tid == 0) { w.ctl->ngrp_l = gl; w.ctl->ngrp_u = gu; }
-  } else {
-    ncl = build_stream<T>(w, P, false, nll, sh);
-    ncu = build_stream<T>(w, P, true, nlu, sh);
-    if (tid == 0) { w.ctl->ngrp_l = nll; w.ctl->ngrp_u = nlu; }
-  }
+}
+
+// Level by level from chunk streams.
+template <typename T>
+__device__ __noinline__ void level_streams(const Walker& w, const Params& P, int nll, int nlu, Shared& sh) {
+  const int tid = threadIdx.x;
+  const int ncl = build_stream<T>(w, P, false, nll, sh);
+  const int ncu = build_stream<T>(w, P, true, nlu, sh);
   if (tid == 0) {
-    w.ctl->nchunk_l = ncl;
-    w.ctl->nchunk_u = ncu;
-    w.ctl->stream_bytes = (ncl ? (long long)w.lchunk[ncl - 1].x + w.lchunk[ncl - 1].y : 0) +
-                          (ncu ? (long long)w.uchunk[ncu - 1].x + w.uchunk[ncu - 1].y : 0);
+    Ctl* c = w.ctl;
+    c->tri_tasks = 0;
+    c->ngrp_l = nll;
+    c->ngrp_u = nlu;
+    c->nchunk_l = ncl;
+    c->nchunk_u = ncu;
+    c->stream_bytes = (ncl ? (long long)w.lchunk[ncl - 1].x + w.lchunk[ncl - 1].y : 0) +
+                      (ncu ? (long long)w.uchunk[ncu - 1].x + w.uchunk[ncu - 1].y : 0);
+  }
+}
+
+// Block-wide: relabel U columns to factor labels, compute U levels (warp 0, reverse
+// order) and build the streams of the triangular solves.
+template <typename T>
+__device__ __noinline__ void relabel_and_levels(const Walker& w, const Params& P, Shared& sh) {
+  const int n = w.n, tid = threadIdx.x, nt = blockDim.x, capLU = w.capLU;
+  for (int idx = tid; idx < n * capLU; idx += nt) {
+    const int r = idx / capLU, t = idx - r * capLU;
+    if (t < w.u_len[r]) w.u_col[idx] = w.iperm[w.u_col[idx]];
+  }
+  __syncthreads();
+  if (tid < 32) {
+    // rows from the last up: a row's level waits for the rows it reads, so its columns are
+    // loaded kAhead rows earlier and the levels kept in shared memory where they fit
+    constexpr int kAhead = 4;
+    const int lane = tid;
+    int* lev = (size_t)4 * n <= (size_t)P.dsm_bytes ? (int*)dyn_smem() : w.lev_u;
+    int ul[kAhead], c0[kAhead], c1[kAhead];
+    auto load = [&](int r, int k) {
+      ul[k] = r >= 0 ? w.u_len[r] : 0;
+      c0[k] = r >= 0 && lane < capLU ? w.u_col[(size_t)r * capLU + lane] : 0;
+      c1[k] = r >= 0 && lane + 32 < capLU ? w.u_col[(size_t)r * capLU + lane + 32] : 0;
+    };
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) load(n - 1 - k, k);
+    for (int r0 = n - 1; r0 >= 0; r0 -= kAhead) {
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k) {
+        const int r = r0 - k;
+        if (r < 0) break;
+        int lv = -1;
+        if (lane < ul[k]) lv = lev[c0[k]];
+        if (lane + 32 < ul[k]) lv = max(lv, lev[c1[k]]);
+        for (int t = lane + 64; t < ul[k]; t += 32) lv = max(lv, lev[w.u_col[(size_t)r * capLU + t]]);
+        lv = __reduce_max_sync(0xffffffffu, lv);
+        if (lane == 0) lev[r] = lv + 1;
+        load(r - kAhead, k);
+        __syncwarp();
+      }
+    }
+    if (lev != w.lev_u)
+      for (int r = lane; r < n; r += 32) w.lev_u[r] = lev[r];
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // scratch is reused by bulk copies
+  }
+  __syncthreads();
+  // level counts
+  int mlv = 0, muv = 0;
+  for (int r = tid; r < n; r += nt) { mlv = max(mlv, w.lev_l[r]); muv = max(muv, w.lev_u[r]); }
+  const int nll = block_max_int(mlv, sh) + 1;
+  const int nlu = block_max_int(muv, sh) + 1;
+  if (tid == 0) { w.ctl->nlev_l = nll; w.ctl->nlev_u = nlu; }
+  const bool tasks = task_solves<T>(w, P);
+  if (!tasks || P.tri_group <= 1) level_sets(w, nll, nlu);
+  if (tasks && build_tasks<T>(w, P, sh)) {
+    if (tid == 0) {
+      w.ctl->tri_tasks = 1;
+      w.ctl->ngrp_l = P.tri_group > 1 ? w.ctl->nchunk_l : nll;
+      w.ctl->ngrp_u = P.tri_group > 1 ? w.ctl->nchunk_u : nlu;
+    }
+  } else {
+    if (tasks && P.tri_group > 1) level_sets(w, nll, nlu);
+    level_streams<T>(w, P, nll, nlu, sh);
   }
   fence_proxy_async_global();  // the streams are read next by bulk (async-proxy) copies
   __syncthreads();

@@ -1,0 +1,76 @@
+"""The task streams of the triangular solves (blocked and level by level) against dense
+triangular solves with the engine's own factors, at the edges of their layout: systems
+smaller than a block, last blocks of one row and of a few, block sizes from 16 to 128 rows,
+CTAs of 2 to 8 warps, two tasks in flight instead of four, and the chunk streams that serve
+what the tasks do not.
+
+Tolerance: with B the rows of a block, an explicit inverse of a diagonal block multiplies the
+rounding of substitution by at most its row sums, a few tens here; 64 rounding errors of a
+row of at most 128 terms at growth 16 give 1e5 eps relative to the largest entry of the
+result (2e-11 FP64, 6e-3 FP32).  The bounds below, 1e-12 and 1e-5, are those of the existing
+apply tests."""
+import numpy as np
+import pytest
+
+import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def vmc():
+    import torch
+
+    assert torch.cuda.is_available()
+    from paper_1008_5113_gb300.build import build_library
+
+    build_library()
+    O.build()
+    from paper_1008_5113_gb300 import vmc as v
+
+    return v
+
+
+CASES = [  # K, lattice, walkers, parameters
+    (3, 0, 1, {}),                                       # 27 rows: one short block
+    (5, 0, 1, {}),                                       # 125 = 64 + 61
+    (4, 0, 1, dict(trisolve_group=2)),                   # 64 = 4 x 16
+    (6, 0, 1, dict(trisolve_group=3)),                   # 216 = 9 x 24
+    (6, 0, 1, dict(trisolve_group=64)),                  # blocks of 128 rows
+    (9, 0, 1, {}),                                       # 729 = 11 x 64 + 25
+    (4, 1, 1, dict(lfil_extra=0)),                       # bcc, 128 rows, factors without fill
+    (6, 0, 1, dict(block_threads=64)),                   # two warps
+    (7, 0, 1, dict(block_threads=160, lfil_extra=40)),   # five warps, long rows
+    (6, 0, 1, dict(trisolve_group=1)),                   # a step per level
+    (7, 0, 1, dict(trisolve_group=0, block_threads=96)),
+    (6, 0, 1, dict(trisolve_group=1, trisolve_warp_rows=8)),  # chunk streams
+    (6, 0, 1, dict(trisolve=1)),                         # synchronisation-free
+    (8, 0, 160, {}),                                     # two CTAs an SM
+    (16, 0, 1, dict(lfil_extra=4)),                      # 4096 rows: larger blocks
+]
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("K,lat,walkers,kw", CASES)
+def test_apply_matches_dense_solves(vmc, prec, K, lat, walkers, kw):
+    a, kappa, rc = (1.0, 2.0, 1.45) if lat == 0 else (2.031, 1.0, 3.39)
+    s = O.system(K, lat, a, kappa, rc)
+    R = O.initial_positions(s, 5, 0.2 * a)
+    n = len(R)
+    ctx = vmc.vmc_create([(K, lat, a, kappa, rc)] * walkers, vmc.params(precision=prec, **kw))
+    try:
+        vmc.vmc_set_positions(ctx, walkers - 1, R)
+        L, U, perm = vmc.vmc_get_factors(ctx, walkers - 1)
+        st = vmc.vmc_get_stats(ctx, walkers - 1)
+        v = np.random.default_rng(K).standard_normal(n)
+        z = vmc.vmc_apply_preconditioner(ctx, walkers - 1, v)
+    finally:
+        vmc.vmc_destroy(ctx)
+    ref = np.zeros(n)
+    ref[perm] = np.linalg.solve(U, np.linalg.solve(L, v))
+    tol = 1e-12 if prec == 0 else 1e-5
+    assert np.abs(z - ref).max() <= tol * np.abs(ref).max()
+    if kw.get("trisolve_group", 8) > 1 and "trisolve" not in kw:
+        assert st["groups_L"] <= 2 * -(-n // 16) and st["groups_U"] <= 2 * -(-n // 16)
+    else:
+        assert st["groups_L"] == st["levels_L"] and st["groups_U"] == st["levels_U"]
