@@ -153,6 +153,7 @@ struct vmc_ctx {
   char* arena = nullptr;
   size_t arena_bytes = 0;
   size_t smem = 0;
+  size_t smem_full = 0;  // ... of a walker CTA alone on its SM
   int64_t sweeps = 0;
   std::string err;
   long long total_n = 0;
@@ -199,6 +200,18 @@ static vmc_status cuda_fail(vmc_ctx* c, cudaError_t e, const char* what) {
   } while (0)
 
 static LaunchCfg cfg(const vmc_ctx* c) { return LaunchCfg{c->stream, c->threads, c->fp64, c->smem}; }
+// Set-up and refactorisation launches: from n = 1024 on a walker's rows in flight need the
+// shared memory of a whole SM (n = 4096: seven warps' rows instead of two when walkers share
+// it), so these run one CTA an SM even where the sweeps run two.
+static LaunchCfg factor_cfg(const vmc_ctx* c, Params& P) {
+  LaunchCfg L = cfg(c);
+  P = c->P;
+  if (c->max_n > 1024 && c->smem_full > L.smem) {
+    L.smem = c->smem_full;
+    P.dsm_bytes = (int)c->smem_full;
+  }
+  return L;
+}
 
 // Automatic background refactorisation (refactor_lag = -1) needs every walker pair on
 // the GPU at once, and systems small enough that a factorisation by one warp finishes
@@ -575,6 +588,7 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     plan_smem(ybytes, budget, ctx->P, p.trisolve == 1);
     if (!ctx->P.y_smem && ybytes != ybytes1) plan_smem(ybytes1, budget, ctx->P, p.trisolve == 1);
     ctx->smem = (size_t)ctx->P.dsm_bytes;
+    ctx->smem_full = (size_t)budget1;
   }
   const size_t ctl_off = cv.take<Ctl>(n_walkers);
   const size_t walk_off = cv.take<Walker>(n_walkers);
@@ -792,7 +806,11 @@ static vmc_status check_walker_status(vmc_ctx* ctx) {
 
 static vmc_status setup_all(vmc_ctx* ctx, int w0, int nwalk) {
   if (ctx->dense) CK(launch_dense_setup(cfg(ctx), ctx->dW + w0, nwalk), "dense setup kernel");
-  else CK(launch_setup(cfg(ctx), ctx->dW, w0, nwalk, ctx->P), "setup kernel");
+  else {
+    Params P;
+    const LaunchCfg L = factor_cfg(ctx, P);
+    CK(launch_setup(L, ctx->dW, w0, nwalk, P), "setup kernel");
+  }
   for (int w = w0; w < w0 + nwalk; ++w) ctx->pending[w] = 0;
   ctx->ready = true;
   return check_walker_status(ctx);
@@ -1249,7 +1267,9 @@ extern "C" vmc_status vmc_refactor(vmc_ctx* ctx, int walker, int reorder) {
   if (ctx && ctx->dense) return fail(ctx, VMC_ERR_INVALID, "not available with the dense engine");
   if (!ctx || walker < 0 || walker >= ctx->nw) return fail(ctx, VMC_ERR_INVALID, "bad arguments");
   if (!ctx->ready) return fail(ctx, VMC_ERR_STATE, "positions not set");
-  CK(launch_refactor(cfg(ctx), ctx->dW, walker, ctx->P, reorder), "refactor kernel");
+  Params P;
+  const LaunchCfg L = factor_cfg(ctx, P);
+  CK(launch_refactor(L, ctx->dW, walker, P, reorder), "refactor kernel");
   ctx->pending[walker] = 0;
   return check_walker_status(ctx);
 }

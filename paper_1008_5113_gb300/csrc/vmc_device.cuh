@@ -213,6 +213,8 @@ struct __align__(16) Shared {
   double cupd[kMaxUpd];
   int alen, ulen;
   int iflag[12];
+  int ilu_done, ilu_lost, ilu_flags, ilu_npiv;  // rows in flight (vmc_ilutp.cuh)
+  long long ilu_nnz;
   double dflag[8];
 };
 

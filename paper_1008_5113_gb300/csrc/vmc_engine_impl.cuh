@@ -666,6 +666,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_setup(const Walker* __restri
   const int fl = factor_block<T>(w, P, sh, true);
   if (lane == 0 && bad) c->status = ST_CAPACITY;
   if (threadIdx.x == 0 && (fl & 2)) c->status = ST_CAPACITY;
+  if (threadIdx.x == 0 && sh.iflag[3]) c->status = ST_TIMEOUT;
 }
 
 template <typename T>
@@ -674,6 +675,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_refactor(const Walker* __res
   ring_init(sh, P);
   const Walker& w = active_of(W[wi]);
   factor_block<T>(w, P, sh, reorder != 0);
+  if (threadIdx.x == 0 && sh.iflag[3]) w.ctl->status = ST_TIMEOUT;
 }
 
 // z = M v for the test entry point: v in r64 (FP64), result in x64 (FP64).

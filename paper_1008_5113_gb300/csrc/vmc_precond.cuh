@@ -1,5 +1,5 @@
 // vmc_precond.cuh -- preconditioner construction on the device:
-//   * the geometric particle/orbital reordering of Sec. 3.1 (greedy rule),
+//   * the geometric particle/orbital reordering of Sec. 3.1 (vmc_reorder.cuh),
 //   * ILUTP (Saad 1994; the threshold/pivoting variant the paper uses in Sec. 4):
 //     row-wise IKJ elimination of A_p with dropping |w_j| < tau ||a_i||_2, at most
 //     nl(i)+p entries kept in the L part and nu(i)+p in the U part, and a column
@@ -8,148 +8,18 @@
 //   * level sets of L and U for the parallel triangular solves.
 #pragma once
 #include "vmc_blocks.cuh"
-#include "vmc_geom.cuh"
+#include "vmc_ilutp.cuh"
+#include "vmc_reorder.cuh"
 
 namespace vmc {
 
-// ---------------------------------------------------------------------------
-// Greedy reordering (Sec. 3.1): for i = 0..n-2, find the orbital nearest to the
-// particle at position i among positions >= i and swap it into column i; if the
-// nearest is already at i, find the particle nearest to orbital i among positions
-// >= i and swap it into row i.  Ties go to the lowest position.  Positions are the
-// current columns; afterwards orbitals return to their fixed columns carrying their
-// new partner particle, so only part_of_row / row_of_part change.
-// Block-wide; O(n^2) distance evaluations.
-// ---------------------------------------------------------------------------
-static __device__ __noinline__ void reorder_block(const Walker& w, Shared& sh) {
-  const int n = w.n, tid = threadIdx.x, nt = blockDim.x;
-  for (int c = tid; c < n; c += nt) { w.gP[c] = w.part_of_row[c]; w.gQ[c] = w.orb_of_col[c]; }
-  __syncthreads();
-  for (int i = 0; i < n - 1; ++i) {
-    const int p = w.gP[i];
-    const double rp[3] = {w.R[3 * p], w.R[3 * p + 1], w.R[3 * p + 2]};
-    double bd = 1e300;
-    int bj = 0x7fffffff;
-    for (int j = i + tid; j < n; j += nt) {
-      const double d = dist2(rp, w.Z + 3 * w.gQ[j], w.L);
-      if (d < bd) { bd = d; bj = j; }
-    }
-    block_argmin(bd, bj, sh);
-    if (bj != i) {
-      if (tid == 0) { const int t = w.gQ[i]; w.gQ[i] = w.gQ[bj]; w.gQ[bj] = t; }
-    } else {
-      const int o = w.gQ[i];
-      const double* zo = w.Z + 3 * o;
-      double bd2 = 1e300;
-      int bk = 0x7fffffff;
-      for (int k = i + tid; k < n; k += nt) {
-        const int q = w.gP[k];
-        const double d = dist2(w.R + 3 * q, zo, w.L);
-        if (d < bd2) { bd2 = d; bk = k; }
-      }
-      block_argmin(bd2, bk, sh);
-      if (bk != i && tid == 0) { const int t = w.gP[i]; w.gP[i] = w.gP[bk]; w.gP[bk] = t; }
-    }
-    __syncthreads();
-  }
-  for (int g = tid; g < n; g += nt) {
-    const int c = w.col_of_orb[w.gQ[g]];
-    const int p = w.gP[g];
-    w.part_of_row[c] = p;
-    w.row_of_part[p] = c;
-  }
-  __syncthreads();
-}
-
-// Top-k of the compacted candidates sh.selF/selV[0..c) by magnitude (ties: smaller
-// label), by one warp: a histogram of binary exponents below the largest one (bins
-// of one octave, the last bin collecting everything smaller) finds the octave that
-// holds the k-th largest; entries in higher octaves are kept, entries in that octave
-// are ranked among themselves.  Result in sh.selK[0..c).
-template <typename W>
-__device__ __forceinline__ int octave_bin(W v, int emax) {
-  int e;
-  frexp(v, &e);
-  return min(63, max(0, emax - e));
-}
+// select_topk of the compacted candidates sh.selF/selV[0..c)
 template <typename W>
 __device__ void select_topk(Shared& sh, int c, int keep) {
-  const int lane = threadIdx.x & 31;
   const W* sv = reinterpret_cast<const W*>(sh.selV);
-  if (c <= keep) {
-    for (int e = lane; e < c; e += 32) sh.selK[e] = 1;
-    __syncwarp();
-    return;
-  }
-  W vmax = 0;
-  for (int e = lane; e < c; e += 32) vmax = fmax(vmax, fabs(sv[e]));
-#pragma unroll
-  for (int o = 16; o; o >>= 1) vmax = fmax(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
-  int emax;
-  frexp(vmax, &emax);
-  for (int b = lane; b < 64; b += 32) sh.hist[b] = 0;
-  __syncwarp();
-  for (int e = lane; e < c; e += 32) atomicAdd(&sh.hist[octave_bin<W>(fabs(sv[e]), emax)], 1);
-  __syncwarp();
-  // boundary bin bb: count(bins < bb) < keep <= count(bins <= bb)
-  int h0 = sh.hist[lane], h1 = sh.hist[lane + 32];
-  int inc0 = h0;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, inc0, o); if (lane >= o) inc0 += v; }
-  const int tot0 = __shfl_sync(0xffffffffu, inc0, 31);
-  int inc1 = h1;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, inc1, o); if (lane >= o) inc1 += v; }
-  inc1 += tot0;
-  const unsigned m0 = __ballot_sync(0xffffffffu, inc0 >= keep);
-  const unsigned m1 = __ballot_sync(0xffffffffu, inc1 >= keep);
-  const int bb = m0 ? __ffs(m0) - 1 : 32 + __ffs(m1) - 1;
-  const int below = (bb < 32 ? __shfl_sync(0xffffffffu, inc0 - h0, bb & 31)
-                             : __shfl_sync(0xffffffffu, inc1 - h1, bb & 31));
-  const int need = keep - below;  // entries to keep from the boundary bin
-  // compact the boundary octave, decide the others
-  int cb = 0;
-  for (int base = 0; base < c; base += 32) {
-    const int e = base + lane;
-    int b = 64;
-    if (e < c) {
-      b = octave_bin<W>(fabs(sv[e]), emax);
-      sh.selK[e] = b < bb ? 1 : 0;
-    }
-    const unsigned m = __ballot_sync(0xffffffffu, b == bb);
-    const int slot = cb + __popc(m & lanemask_lt());
-    if (b == bb && slot < 256) sh.bndE[slot] = e;
-    cb += __popc(m);
-  }
-  __syncwarp();
-  if (cb <= 256) {
-    for (int q = lane; q < cb; q += 32) {
-      const int e = sh.bndE[q];
-      const W me = fabs(sv[e]);
-      const int fe = sh.selF[e];
-      int rank = 0;
-      for (int o = 0; o < cb; ++o) {
-        const int eo = sh.bndE[o];
-        const W mo = fabs(sv[eo]);
-        rank += (mo > me) || (mo == me && sh.selF[eo] < fe);
-      }
-      sh.selK[e] = rank < need ? 1 : 0;
-    }
-  } else {
-    for (int e = lane; e < c; e += 32) {
-      const W me = fabs(sv[e]);
-      if (octave_bin<W>(me, emax) != bb) continue;
-      const int fe = sh.selF[e];
-      int rank = 0;
-      for (int o = 0; o < c; ++o) {
-        const W mo = fabs(sv[o]);
-        if (octave_bin<W>(mo, emax) != bb) continue;
-        rank += (mo > me) || (mo == me && sh.selF[o] < fe);
-      }
-      sh.selK[e] = rank < need ? 1 : 0;
-    }
-  }
-  __syncwarp();
+  using K = decltype(mag_key(W(0)));
+  select_topk<K>(sh.hist, sh.bndE, sh.selK, c, keep, [&](int e) { return mag_key(sv[e]); },
+                 [&](int e) { return sh.selF[e]; });
 }
 
 // ---------------------------------------------------------------------------
@@ -1059,6 +929,39 @@ __device__ int build_stream(const Walker& w, const Params& P, bool upper, int nl
   return nch_total;
 }
 
+// One warp: the level of every row, 1 + the largest of the rows it reads (0 without any); U
+// (up) from the last row up.  A row's level waits for the rows it reads, so its columns are
+// loaded kAhead rows earlier.
+static __device__ __noinline__ void row_levels(const int* len, const int* col, int n, int capLU, bool up, int* lev) {
+  constexpr int kAhead = 4;
+  const int lane = threadIdx.x & 31;
+  int L[kAhead], c0[kAhead], c1[kAhead];
+  auto row = [&](int i) { return up ? n - 1 - i : i; };
+  auto load = [&](int i, int k) {
+    const size_t b = (size_t)(i < n ? row(i) : 0) * capLU;
+    L[k] = i < n ? len[row(i)] : 0;
+    c0[k] = i < n && lane < capLU ? col[b + lane] : 0;
+    c1[k] = i < n && lane + 32 < capLU ? col[b + lane + 32] : 0;
+  };
+#pragma unroll
+  for (int k = 0; k < kAhead; ++k) load(k, k);
+  for (int i0 = 0; i0 < n; i0 += kAhead) {
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) {
+      const int i = i0 + k;
+      if (i >= n) break;
+      int lv = -1;
+      if (lane < L[k]) lv = lev[c0[k]];
+      if (lane + 32 < L[k]) lv = max(lv, lev[c1[k]]);
+      for (int t = lane + 64; t < L[k]; t += 32) lv = max(lv, lev[col[(size_t)row(i) * capLU + t]]);
+      lv = __reduce_max_sync(0xffffffffu, lv);
+      if (lane == 0) lev[row(i)] = lv + 1;
+      load(i + kAhead, k);
+      __syncwarp();
+    }
+  }
+}
+
 // Packs both level sets (counting sort by level).  Block-wide, ends synchronised.
 static __device__ __noinline__ void level_sets(const Walker& w, int nll, int nlu) {
   const int n = w.n, tid = threadIdx.x, nt = blockDim.x;
@@ -1103,8 +1006,8 @@ __device__ __noinline__ void level_streams(const Walker& w, const Params& P, int
   }
 }
 
-// Block-wide: relabel U columns to factor labels, compute U levels (warp 0, reverse
-// order) and build the streams of the triangular solves.
+// Block-wide: relabel U columns to factor labels, compute the levels and build the streams
+// of the triangular solves.
 template <typename T>
 __device__ __noinline__ void relabel_and_levels(const Walker& w, const Params& P, Shared& sh) {
   const int n = w.n, tid = threadIdx.x, nt = blockDim.x, capLU = w.capLU;
@@ -1113,37 +1016,14 @@ __device__ __noinline__ void relabel_and_levels(const Walker& w, const Params& P
     if (t < w.u_len[r]) w.u_col[idx] = w.iperm[w.u_col[idx]];
   }
   __syncthreads();
-  if (tid < 32) {
-    // rows from the last up: a row's level waits for the rows it reads, so its columns are
-    // loaded kAhead rows earlier and the levels kept in shared memory where they fit
-    constexpr int kAhead = 4;
-    const int lane = tid;
-    int* lev = (size_t)4 * n <= (size_t)P.dsm_bytes ? (int*)dyn_smem() : w.lev_u;
-    int ul[kAhead], c0[kAhead], c1[kAhead];
-    auto load = [&](int r, int k) {
-      ul[k] = r >= 0 ? w.u_len[r] : 0;
-      c0[k] = r >= 0 && lane < capLU ? w.u_col[(size_t)r * capLU + lane] : 0;
-      c1[k] = r >= 0 && lane + 32 < capLU ? w.u_col[(size_t)r * capLU + lane + 32] : 0;
-    };
-#pragma unroll
-    for (int k = 0; k < kAhead; ++k) load(n - 1 - k, k);
-    for (int r0 = n - 1; r0 >= 0; r0 -= kAhead) {
-#pragma unroll
-      for (int k = 0; k < kAhead; ++k) {
-        const int r = r0 - k;
-        if (r < 0) break;
-        int lv = -1;
-        if (lane < ul[k]) lv = lev[c0[k]];
-        if (lane + 32 < ul[k]) lv = max(lv, lev[c1[k]]);
-        for (int t = lane + 64; t < ul[k]; t += 32) lv = max(lv, lev[w.u_col[(size_t)r * capLU + t]]);
-        lv = __reduce_max_sync(0xffffffffu, lv);
-        if (lane == 0) lev[r] = lv + 1;
-        load(r - kAhead, k);
-        __syncwarp();
-      }
-    }
-    if (lev != w.lev_u)
-      for (int r = lane; r < n; r += 32) w.lev_u[r] = lev[r];
+  // levels of both factors, a warp each; in shared memory where they fit
+  if (tid < 64) {
+    const bool up = tid < 32, sm = (size_t)8 * n <= (size_t)P.dsm_bytes;
+    int* glob = up ? w.lev_u : w.lev_l;
+    int* lev = sm ? (int*)dyn_smem() + (up ? 0 : n) : glob;
+    row_levels(up ? w.u_len : w.l_len, up ? w.u_col : w.l_col, n, capLU, up, lev);
+    if (sm)
+      for (int r = tid & 31; r < n; r += 32) glob[r] = lev[r];
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // scratch is reused by bulk copies
   }
   __syncthreads();
@@ -1175,32 +1055,36 @@ template <typename T>
 __device__ __noinline__ int factor_block(const Walker& w, const Params& P, Shared& sh, bool reorder) {
   const long long t0 = clock64();
   if (reorder) {
-    reorder_block(w, sh);
+    reorder_block(w, P);
     if (threadIdx.x == 0) w.ctl->cyc[PH_REORDER] += clock64() - t0;
   }
-  if (threadIdx.x < 32) {
-    int npiv = 0, p = 0;
-    double nnz = 0.0;
-    for (int r = threadIdx.x; r < w.n; r += 32) w.lev_u[r] = 0;
-    const long long ti = clock64();
-    int fl;
+  const long long ti = clock64();
+  int npiv = 0, p = 0, fl = 0;
+  double nnz = 0.0;
+  // rows in flight on several warps where at least two warps' working rows fit shared memory;
+  // else one warp: the hashed working row where the dense one does not fit shared memory
+  // (n > 6000 or so, or forced), else the dense row
+  const PipePlan pp = P.ilu64 ? ilu_pipe_plan<double>(w.n, (size_t)P.dsm_bytes, blockDim.x >> 5)
+                              : ilu_pipe_plan<T>(w.n, (size_t)P.dsm_bytes, blockDim.x >> 5);
+  if (pp.warps >= 2 && P.ilu_variant != 2 && w.ex_val != nullptr && w.u_head != nullptr) {
+    fl = P.ilu64 ? ilutp_pipe<double>(w, P, sh, pp, w.ex_val, &npiv, &nnz, &p)
+                 : ilutp_pipe<T>(w, P, sh, pp, (T*)w.ex_val, &npiv, &nnz, &p);
+  } else if (threadIdx.x < 32) {
     const IluSm pl64 = ilu_sm_plan<double>(w.n, (size_t)P.dsm_bytes);
     const IluSm plT = ilu_sm_plan<T>(w.n, (size_t)P.dsm_bytes);
-    // the shared-memory variant where the dense working row does not fit in shared memory
-    // (about n > 6000 with one walker CTA per SM); below that the dense row is in shared
-    // memory too and, with its U-row cache, the faster of the two
     const bool dense_row_in_smem = 4 * (size_t)(pad4((w.n + 31) >> 5) + pad4((((w.n + 31) >> 5) + 31) >> 5)) +
                                        16 + (size_t)16 * w.n <= (size_t)P.dsm_bytes;
-    if (P.ilu_variant == 0 && !dense_row_in_smem && w.u_head != nullptr && (P.ilu64 ? pl64.ok : plT.ok))
-      fl = P.ilu64 ? ilutp_warp_hash<double>(w, P, sh, pl64, &npiv, &nnz, &p)
-                   : ilutp_warp_hash<T>(w, P, sh, plT, &npiv, &nnz, &p);
-    else if (P.ilu_variant == 2 && w.u_head != nullptr && (P.ilu64 ? pl64.ok : plT.ok))  // forced (tests)
+    const bool hash = (P.ilu_variant == 2 || (P.ilu_variant == 0 && !dense_row_in_smem)) && w.u_head != nullptr &&
+                      (P.ilu64 ? pl64.ok : plT.ok);
+    if (hash)
       fl = P.ilu64 ? ilutp_warp_hash<double>(w, P, sh, pl64, &npiv, &nnz, &p)
                    : ilutp_warp_hash<T>(w, P, sh, plT, &npiv, &nnz, &p);
     else
       fl = P.ilu64 ? ilutp_warp<double>(w, P, sh, &npiv, &nnz, &p) : ilutp_warp<T>(w, P, sh, &npiv, &nnz, &p);
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // scratch is reused by bulk copies
+  if (threadIdx.x < 32) {
     if (threadIdx.x == 0) w.ctl->cyc[PH_ILUTP] += clock64() - ti;
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // scratch is reused by bulk copies
     if (threadIdx.x == 0) {
       sh.iflag[0] = fl;
       Ctl* c = w.ctl;
@@ -1216,15 +1100,18 @@ __device__ __noinline__ int factor_block(const Walker& w, const Params& P, Share
     }
   }
   __syncthreads();
-  const int fl = sh.iflag[0];
+  fl = sh.iflag[0];
   const long long tl = clock64();
   relabel_and_levels<T>(w, P, sh);
   if (threadIdx.x == 0) w.ctl->cyc[PH_LEVELS] += clock64() - tl;
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 32) {
     long long tot = 0;
-    for (int i = 0; i < w.n; ++i) tot += w.a_len[i];
-    w.ctl->nnz_A = (double)tot;
-    w.ctl->cyc[PH_FACTOR] += clock64() - t0;
+    for (int i = threadIdx.x; i < w.n; i += 32) tot += w.a_len[i];
+    tot = warp_sum_ll(tot);
+    if (threadIdx.x == 0) {
+      w.ctl->nnz_A = (double)tot;
+      w.ctl->cyc[PH_FACTOR] += clock64() - t0;
+    }
   }
   __syncthreads();
   return fl;
