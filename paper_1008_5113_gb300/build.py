@@ -1,6 +1,6 @@
 """In-tree build of the CUDA library ``libvmc.so`` for sm_103a (nvcc, no cmake).
 
-The translation units (the engine's kernels in FP64 and in FP32, the precision-independent
+The translation units (the engine's kernels in FP64 and in FP32, in six parts each, the precision-independent
 launch entry points; C ABI + host layout; the allocation-free entry point; the dense
 reference engine) compile in parallel and are linked into
 ``paper_1008_5113_gb300/libvmc.so`` next to this file.
@@ -17,7 +17,10 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libvmc.so")
 GENCODE = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["vmc_engine_f64.cu", "vmc_engine_f32.cu", "vmc_engine.cu", "vmc_capi.cu", "vmc_noalloc.cu", "vmc_dense.cu"]
+# (source, defines): the engine's kernels are compiled in parts, the longest first
+PARTS = [2, 1, 3, 4, 0, 5]
+SOURCES = [(f"vmc_engine_{p}.cu", [f"-DVMC_PART={k}"]) for k in PARTS for p in ("f32", "f64")]
+SOURCES += [(s, []) for s in ("vmc_engine.cu", "vmc_capi.cu", "vmc_noalloc.cu", "vmc_dense.cu")]
 
 
 def _nvcc() -> str:
@@ -48,10 +51,10 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
     common = ["-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-lineinfo", *GENCODE, "-I", os.path.join(ROOT, "include")]
     with tempfile.TemporaryDirectory(prefix="vmcbuild") as tmp:
         procs, objs = [], []
-        for src in SOURCES:
-            obj = os.path.join(tmp, src + ".o")
+        for src, defs in SOURCES:
+            obj = os.path.join(tmp, src + "".join(defs) + ".o")
             objs.append(obj)
-            cmd = [nvcc, *common, "-c", os.path.join(CSRC, src), "-o", obj]
+            cmd = [nvcc, *common, *defs, "-c", os.path.join(CSRC, src), "-o", obj]
             if verbose:
                 print(" ".join(cmd), flush=True)
             procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))

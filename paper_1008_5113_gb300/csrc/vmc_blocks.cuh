@@ -58,8 +58,9 @@ __device__ __forceinline__ void values_from(const unsigned char* p, double* q) {
 
 __device__ __forceinline__ void bar_all() { asm volatile("bar.sync 0;" ::: "memory"); }
 
-template <typename T, int D>
+template <typename T>
 __device__ __forceinline__ void run_tasks(const Walker& w, const Params& P, const T* v, T* vec) {
+  const int D = tasks_ahead<T>(P) >= 4 ? 4 : 2;  // tasks in flight
   constexpr int TB = task_bytes((int)sizeof(T));
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int2 tl = w.lchunk[wid], tu = w.uchunk[wid];
@@ -81,14 +82,15 @@ __device__ __forceinline__ void run_tasks(const Walker& w, const Params& P, cons
     }
     cp_commit();
   };
-#pragma unroll
+#pragma unroll 1
   for (int d = 0; d < D; ++d) issue(d, d, 32);
-  block_copy(vec, v, w.n);
+  if (v) block_copy(vec, v, w.n);  // else v is in the solve vector already
   unsigned word = 0;
   uint4 c = make_uint4(0u, 0u, 0u, 0u);
   T q[kLaneEntries];
   auto fetch = [&](int slot) {  // the task that has landed in slot, into registers
-    cp_wait<D - 1>();
+    if (D == 4) cp_wait<3>();
+    else cp_wait<1>();
     __syncwarp();
     const unsigned char* p = ring + slot * TB;
     word = *reinterpret_cast<const unsigned*>(p + 4 * lane);
@@ -98,10 +100,13 @@ __device__ __forceinline__ void run_tasks(const Walker& w, const Params& P, cons
   };
   if (nt > 0) fetch(0);
   __syncthreads();
+#pragma unroll 1
   for (int i = 0; i < lead_l; ++i) bar_all();
   int slot = 0;
+#pragma unroll 1
   for (int t = 0; t < nt; ++t) {
     if (t == nl)
+#pragma unroll 1
       for (int i = 0; i < lead_u; ++i) bar_all();
     const int after = (int)((word >> 16) & 31u), nb = (int)((word >> 22) & 15u), dst = (int)(word & 0xffffu);
     const bool first = (word & (1u << 21)) != 0;
@@ -114,14 +119,17 @@ __device__ __forceinline__ void run_tasks(const Walker& w, const Params& P, cons
     issue(t + D, slot, (int)((word >> 26) & 31u) + 1);  // every lane has read the slot: its own part above, the words at the shuffle
     slot = slot + 1 == D ? 0 : slot + 1;
     fetch(slot);
+#pragma unroll 1
     for (int o = 1; o <= widest; o <<= 1) {  // sum over the row's lanes into its first
       const T p2 = __shfl_down_sync(0xffffffffu, part, o);
       if (o <= after) part += p2;
     }
     if (first) vec[dst] = part;
+#pragma unroll 1
     for (int i = 0; i < nb; ++i) bar_all();
   }
   if (nl == nt)  // no task in U's steps
+#pragma unroll 1
     for (int i = 0; i < lead_u; ++i) bar_all();
   __syncthreads();
 }
@@ -132,8 +140,7 @@ __device__ __forceinline__ void run_tasks(const Walker& w, const Params& P, cons
 template <typename T>
 __device__ __forceinline__ T* tri_tasks(const Walker& w, const Params& P, const T* v) {
   T* vec = (T*)dyn_smem();
-  if (tasks_ahead<T>(P) >= 4) run_tasks<T, 4>(w, P, v, vec);
-  else run_tasks<T, 2>(w, P, v, vec);
+  run_tasks<T>(w, P, v, vec);
   return vec;
 }
 
@@ -158,6 +165,7 @@ __device__ __forceinline__ int plan_step(const int (&len)[4], int m, int (&pos)[
   }
   most = warp_max_int(most);
   if (most > 32) return -1;
+#pragma unroll 1
   for (int g = most; g > 0; --g) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -214,6 +222,7 @@ __device__ __noinline__ bool build_tasks(const Walker& w, const Params& P, Share
     return t0 < T_ ? (T_ - 1 - t0) / nw + 1 : 0;
   };
   if (tid == 0) sh.iflag[10] = 0;
+#pragma unroll 1
   for (int upper = 0; upper < 2; ++upper) {
     const int* flen = upper ? w.u_len : w.l_len;
     const int* fcol = upper ? w.u_col : w.l_col;
@@ -226,11 +235,14 @@ __device__ __noinline__ bool build_tasks(const Walker& w, const Params& P, Share
     auto lo_of = [&](int b) { return upper ? max(0, n - (b + 1) * B) : b * B; };
     auto hi_of = [&](int b) { return upper ? n - b * B : min(n, (b + 1) * B); };
     if (by_level) {
+#pragma unroll 1
       for (int l = tid; l < nlev; l += nt) w.lvl_cur[l] = (lptr[l + 1] - lptr[l] + kMaxBlk - 1) / kMaxBlk;
       __syncthreads();
       nst = block_scan_inplace(w.lvl_cur, nlev, sh);  // first step of every level
       if ((size_t)nst * nw > (size_t)room || nst > n) return false;
+#pragma unroll 1
       for (int l = wid; l < nlev; l += nw)
+#pragma unroll 1
         for (int q0 = lptr[l], s = w.lvl_cur[l]; q0 < lptr[l + 1]; q0 += kMaxBlk, ++s) {
           const int m = min(kMaxBlk, lptr[l + 1] - q0);
           int len[4], pos[4];
@@ -255,10 +267,12 @@ __device__ __noinline__ bool build_tasks(const Walker& w, const Params& P, Share
         }
     } else {
       // 1. entries of every row inside its diagonal block: {entry, local column}, and the counts
+#pragma unroll 1
       for (int r = wid; r < n; r += nw) {
         const int b = upper ? (n - 1 - r) / B : r / B;
         const int lo = lo_of(b), hi = hi_of(b), L = flen[r];
         int nin = 0;
+#pragma unroll 1
         for (int t0 = 0; t0 < L; t0 += 32) {
           const int t = t0 + lane;
           const int c = t < L ? fcol[(size_t)r * capLU + t] : -1;
@@ -272,10 +286,12 @@ __device__ __noinline__ bool build_tasks(const Walker& w, const Params& P, Share
       __syncthreads();
       // 2. inverses of the diagonal blocks, a thread per column: X(i, j) of block b at
       //    ex_val[row of i][j]
+#pragma unroll 1
       for (int idx = tid; idx < nb * B; idx += nt) {
         const int b = idx / B, j = idx - b * B;
         const int lo = lo_of(b), hi = hi_of(b), m = hi - lo;
         if (j >= m) continue;
+#pragma unroll 1
         for (int i = 0; i < m; ++i) {
           const int r = upper ? hi - 1 - i : lo + i;
           const double d = upper ? w.u_dinv64[r] : 1.0;
@@ -285,6 +301,7 @@ __device__ __noinline__ bool build_tasks(const Walker& w, const Params& P, Share
           } else if (i > j) {
             const int k = w.ex_len[r];
             double acc = 0.0;
+#pragma unroll 1
             for (int t = 0; t < k; ++t) {
               const int e = w.ex_col[(size_t)r * EX + t], li = e >> 16;
               if (li >= j)
@@ -298,8 +315,10 @@ __device__ __noinline__ bool build_tasks(const Walker& w, const Params& P, Share
       __syncthreads();
       // 3. steps of every block: 2, or 1 when no row has an entry inside its diagonal block (0
       //    for L when there is none outside either)
+#pragma unroll 1
       for (int b = wid; b < nb; b += nw) {
         int in = 0, out = 0;
+#pragma unroll 1
         for (int r = lo_of(b) + lane; r < hi_of(b); r += 32) {
           in |= w.ex_len[r];
           out |= flen[r] - w.ex_len[r];
@@ -308,12 +327,15 @@ __device__ __noinline__ bool build_tasks(const Walker& w, const Params& P, Share
         if (lane == 0) w.lvl_nchunk[b] = any_in ? 2 : (any_out || upper ? 1 : 0);
       }
       __syncthreads();
+#pragma unroll 1
       for (int b = tid; b < nb; b += nt) w.lvl_cur[b] = w.lvl_nchunk[b];
       __syncthreads();
       nst = block_scan_inplace(w.lvl_cur, nb, sh);  // first step of every block
       // 4. lanes of every row
+#pragma unroll 1
       for (int b = wid; b < nb; b += nw) {
         const int lo = lo_of(b), m = hi_of(b) - lo, ns = w.lvl_nchunk[b];
+#pragma unroll 1
         for (int ph = 0; ph < ns; ++ph) {
           int len[4], pos[4];
   #pragma unroll
@@ -327,6 +349,7 @@ __device__ __noinline__ bool build_tasks(const Walker& w, const Params& P, Share
                 len[q] = 1 + flen[r] - w.ex_len[r];
               } else {
                 int k = 0;
+#pragma unroll 1
                 for (int j = 0; j < m; ++j) k += w.ex_val[(size_t)r * EX + j] != 0.0;
                 len[q] = k;
               }
@@ -349,10 +372,12 @@ __device__ __noinline__ bool build_tasks(const Walker& w, const Params& P, Share
     const int before = ntask;
     int lead = nst;
     if (tid < nw) {
+#pragma unroll 1
       for (int s = 0; s < nst; ++s) {
         tbase[(size_t)s * nw + tid] = ntask;
         ntask += warp_tasks(s, tid);
       }
+#pragma unroll 1
       for (int s = nst - 1; s >= 0; --s) {
         tbar[(size_t)s * nw + tid] = lead - s;
         if (warp_tasks(s, tid) > 0) lead = s;
@@ -371,19 +396,24 @@ __device__ __noinline__ bool build_tasks(const Walker& w, const Params& P, Share
     auto bars_after = [&](int s, int t) {
       return (unsigned)(t + nw >= w.chunk_meta[s].w ? tbar[(size_t)s * nw + (t + s) % nw] : 0) << 22;
     };
+#pragma unroll 1
     for (int s = 0; s < nst; ++s)
+#pragma unroll 1
       for (int t = wid; t < w.chunk_meta[s].w; t += nw) {
         unsigned char* base = task_at(s, t);
         ((unsigned*)base)[lane] = bars_after(s, t);
         ((uint4*)(base + 128))[lane] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 1
         for (int k = 0; k < kLaneEntries * tsz / 16; ++k) ((uint4*)(base + 640 + 512 * k))[lane] = make_uint4(0u, 0u, 0u, 0u);
       }
     __syncthreads();
+#pragma unroll 1
     for (int r = wid; r < n; r += nw) {
       const int b = upper ? (n - 1 - r) / B : r / B;
       const int lo = by_level ? r : lo_of(b), hi = by_level ? r + 1 : hi_of(b), m = hi - lo;
       const int ns = by_level ? 1 : w.lvl_nchunk[b], s0 = by_level ? stepof[r] : w.lvl_cur[b];
       const int li = upper ? hi - 1 - r : r - lo;
+#pragma unroll 1
       for (int ph = 0; ph < ns; ++ph) {
         const int s = s0 + ph;
         const int p = (ph == 0 ? posA : posB)[r], l0 = p & 31;
@@ -403,6 +433,7 @@ __device__ __noinline__ bool build_tasks(const Walker& w, const Params& P, Share
           if (lane == 0) put(0, r, d);
           k = 1;
           const int L = flen[r];
+#pragma unroll 1
           for (int t0 = 0; t0 < L; t0 += 32) {
             const int t = t0 + lane;
             const int c = t < L ? fcol[(size_t)r * capLU + t] : -1;
@@ -413,9 +444,11 @@ __device__ __noinline__ bool build_tasks(const Walker& w, const Params& P, Share
           }
         } else {
           int cnt = 0;
+#pragma unroll 1
           for (int j0 = 0; j0 < m; j0 += 32)
             cnt += __popc(__ballot_sync(0xffffffffu, j0 + lane < m && w.ex_val[(size_t)r * EX + j0 + lane] != 0.0));
           G = row_lanes(cnt);
+#pragma unroll 1
           for (int j0 = 0; j0 < m; j0 += 32) {
             const int j = j0 + lane;
             const double xv = j < m ? w.ex_val[(size_t)r * EX + j] : 0.0;
@@ -424,6 +457,7 @@ __device__ __noinline__ bool build_tasks(const Walker& w, const Params& P, Share
             k += __popc(mk);
           }
         }
+#pragma unroll 1
         for (int i = k + lane; i < kLaneEntries * G; i += 32) put(i, self, 0.0);  // padding reads the row's own value
         if (lane < G)
           ((unsigned*)base)[l0 + lane] = (unsigned)dst | ((unsigned)(G - 1 - lane) << 16) | (lane == 0 ? 1u << 21 : 0u) |
@@ -439,6 +473,7 @@ __device__ __noinline__ bool build_tasks(const Walker& w, const Params& P, Share
   {
     const int mine = (w.lchunk[wid].y & 0xffffff) + (w.uchunk[wid].y & 0xffffff);
     unsigned* base = (unsigned*)(w.lstream + (size_t)wid * share);
+#pragma unroll 1
     for (int t = 0; t < mine; ++t) {
       const int lanes = __popc(__ballot_sync(0xffffffffu, base[(size_t)t * (TB / 4) + lane] >> 31));
       used += lanes;

@@ -154,6 +154,7 @@ struct vmc_ctx {
   size_t arena_bytes = 0;
   size_t smem = 0;
   size_t smem_full = 0;  // ... of a walker CTA alone on its SM
+  int per_sm = 1;        // walker CTAs an SM holds
   int64_t sweeps = 0;
   std::string err;
   long long total_n = 0;
@@ -199,7 +200,7 @@ static vmc_status cuda_fail(vmc_ctx* c, cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_fail(ctx, e_, what); \
   } while (0)
 
-static LaunchCfg cfg(const vmc_ctx* c) { return LaunchCfg{c->stream, c->threads, c->fp64, c->smem}; }
+static LaunchCfg cfg(const vmc_ctx* c) { return LaunchCfg{c->stream, c->threads, c->fp64, c->smem, c->per_sm}; }
 // Set-up and refactorisation launches: from n = 1024 on a walker's rows in flight need the
 // shared memory of a whole SM (n = 4096: seven warps' rows instead of two when walkers share
 // it), so these run one CTA an SM even where the sweeps run two.
@@ -450,12 +451,13 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
   const size_t Tsz = ctx->fp64 ? sizeof(double) : sizeof(float);
   const int m = p.gmres_m, mu = std::max(1, p.max_updates);
   std::vector<std::vector<size_t>> offs(n_walkers);
+  std::vector<size_t> ell_off(3 * (size_t)n_walkers);  // transposed slots: columns, FP64, FP32
   Carve cv;
   ctx->hw.resize(n_walkers);
   long long base = 0;
   for (int w = 0; w < n_walkers; ++w) {
     const Layout& L = lay[w];
-    const int n = L.n, cap = L.cap;
+    const int n = L.n, cap = L.cap, ld = pad4(n);
     const int pmax = p.lfil_extra >= 0 ? p.lfil_extra : (cap + 1) / 2;
     const int capLU = (cap + pmax + 2 + 3) / 4 * 4;  // rows of 16-byte multiples (bulk copies)
     const int exmax = expanded_row_cap(capLU, p.trisolve_row_cap);
@@ -468,7 +470,8 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     o.push_back(cv.take<int>(n));                      // 5 part_of_row
     o.push_back(cv.take<int>((size_t)n * cap));        // 6 a_col
     o.push_back(cv.take<double>((size_t)n * cap));     // 7 a_val
-    o.push_back(cv.take<float>((size_t)n * cap));      // 8 a_val32
+    const bool ell = n < 0x10000;
+    o.push_back(cv.take<float>(ell ? 0 : (size_t)n * cap));  // 8 a_val32
     o.push_back(cv.take<int>(n));                      // 9 a_len
     o.push_back(cv.take<int>((size_t)n * capLU));      // 10 l_col
     o.push_back(cv.take<double>((size_t)n * capLU));   // 11 l_val64
@@ -494,13 +497,13 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     o.push_back(cv.take<int>(n));                      // 30 wpos
     o.push_back(cv.take<int>(n));                      // 31 gP
     o.push_back(cv.take<int>(n));                      // 32 gQ
-    o.push_back(cv.take<char>((size_t)((mu + 3) / 4 * 4) * n * Tsz)); // 33 upd_z (transposed)
-    o.push_back(cv.take<int>((size_t)mu * kMaxU));     // 34 upd_ucol
-    o.push_back(cv.take<char>((size_t)mu * kMaxU * Tsz));  // 35 upd_uval
+    o.push_back(cv.take<char>((size_t)mu * ld * Tsz)); // 33 upd_z
+    o.push_back(cv.take<int>((size_t)kMaxUpd * kMaxU));     // 34 upd_ucol
+    o.push_back(cv.take<char>((size_t)kMaxUpd * kMaxU * Tsz));  // 35 upd_uval
     o.push_back(cv.take<int>(mu));                     // 36 upd_ulen
     o.push_back(cv.take<double>((size_t)kMaxUpd * kMaxUpd));  // 37 upd_G
-    o.push_back(cv.take<char>((size_t)(m + 1) * n * Tsz));    // 38 V
-    o.push_back(cv.take<char>((size_t)m * n * Tsz));          // 39 Zk
+    o.push_back(cv.take<char>((size_t)(m + 1) * ld * Tsz));   // 38 V
+    o.push_back(cv.take<char>((size_t)m * ld * Tsz));         // 39 Zk
     o.push_back(cv.take<char>((size_t)3 * n * Tsz));          // 40 tv (three solve vectors)
     o.push_back(cv.take<double>(n));                   // 41 x64
     o.push_back(cv.take<double>(n));                   // 42 r64
@@ -553,10 +556,13 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
       o.push_back(cv.take<int>((size_t)n * exmax));      // ex_col
       o.push_back(cv.take<double>((size_t)n * exmax));   // ex_val
     }
+    ell_off[w] = cv.take<unsigned short>(ell ? (size_t)cap * ld : 0);
+    ell_off[n_walkers + w] = cv.take<double>(ell ? (size_t)cap * ld : 0);
+    ell_off[2 * (size_t)n_walkers + w] = cv.take<float>(ell && !ctx->fp64 ? (size_t)cap * ld : 0);
     Walker& W = ctx->hw[w];
     std::memset(&W, 0, sizeof(W));
     W.n = n; W.K = systems[w].K; W.lattice = systems[w].lattice; W.cap = cap; W.capLU = capLU;
-    W.m = m; W.mu = mu; W.mu4 = (mu + 3) / 4 * 4; W.per = L.per;
+    W.m = m; W.mu = mu; W.ld = ld; W.per = L.per;
     W.a = systems[w].a; W.kappa = systems[w].kappa; W.rc = systems[w].r_c;
     W.rc2 = systems[w].r_c * systems[w].r_c; W.L = systems[w].K * systems[w].a;
     W.log_base = base;
@@ -584,7 +590,10 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     const int budget1 = optin - stat;
     const int budget2 = per_sm / 2 - 1024 - stat;
     int budget = budget1;
-    if (n_walkers > nsm && budget2 >= ybytes + 2 * kSlotBytes) budget = budget2;
+    if (n_walkers > nsm && budget2 >= ybytes + 2 * kSlotBytes) {
+      budget = budget2;
+      ctx->per_sm = 2;
+    }
     plan_smem(ybytes, budget, ctx->P, p.trisolve == 1);
     if (!ctx->P.y_smem && ybytes != ybytes1) plan_smem(ybytes1, budget, ctx->P, p.trisolve == 1);
     ctx->smem = (size_t)ctx->P.dsm_bytes;
@@ -618,7 +627,13 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     W.part_of_row = (int*)(A + o[5]);
     W.a_col = (int*)(A + o[6]);
     W.a_val = (double*)(A + o[7]);
-    W.a_val32 = (float*)(A + o[8]);
+    if (W.n < 0x10000) {
+      W.ell_col = (unsigned short*)(A + ell_off[w]);
+      W.ell_val = (double*)(A + ell_off[n_walkers + w]);
+      if (!ctx->fp64) W.ell_val32 = (float*)(A + ell_off[2 * (size_t)n_walkers + w]);
+    } else {
+      W.a_val32 = (float*)(A + o[8]);
+    }
     W.a_len = (int*)(A + o[9]);
     W.l_col = (int*)(A + o[10]);
     W.l_val64 = (double*)(A + o[11]);

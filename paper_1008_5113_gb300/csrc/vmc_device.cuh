@@ -102,7 +102,7 @@ struct Ctl {
 // Immutable-per-context description of one walker: sizes and device pointers.
 struct Walker {
   int n, K, lattice, cap, capLU, m, mu;
-  int mu4;                // row stride of the transposed z_hat store (mu rounded up to 4)
+  int ld;                 // row stride of V, Zk, the z_hat store and the transposed slots (n rounded up to 4)
   int per;                // sites per cubic cell (1 sc, 2 bcc)
   double a, kappa, rc, rc2, L;
   const double* Z;        // n*3 orbital centres
@@ -111,7 +111,10 @@ struct Walker {
   double* R;              // n*3 positions by particle
   int* row_of_part;
   int* part_of_row;
-  int* a_col; double* a_val; float* a_val32; int* a_len;
+  int* a_col; double* a_val; float* a_val32; int* a_len;  // a_val32: only without the transposed copy
+  // transposed copy of the slots for the products with A (quads of entries: entry t of particle
+  // p at ((t / 4) ld + p) 4 + t % 4; nullptr: n >= 65536, or no room): columns, values in FP64 and, mixed, FP32
+  unsigned short* ell_col; double* ell_val; float* ell_val32;
   int* l_col; double* l_val64; int* l_len;
   int* u_col; double* u_val64; int* u_len;
   double* u_dinv64;
@@ -182,8 +185,18 @@ struct Params {
   long long budget_total;
 };
 
+// What the phases of a solve did, for the statistics (flush_counts).
+struct SolveCounts {
+  int applies, its, sumj, its2, sumj2, cycles, sumx, resid;
+};
+
 // Shared memory of a walker CTA (static, < 48 KB).
 struct __align__(16) Shared {
+  // The walker's view and the parameters: the functions of the solve take them by reference,
+  // and with the solve's data filling the SM's shared memory there is next to no L1 -- a
+  // pointer or a size read from global or local memory costs an L2 round trip (300 cycles).
+  Walker walk;
+  Params par;
   unsigned long long bar[kMaxSlots];  // "full" mbarriers of the stream ring
   unsigned long long ebar[kMaxSlots]; // "empty" mbarriers (released by the consumer warps)
   int ring_seq;                       // chunks consumed so far in this launch
@@ -211,6 +224,10 @@ struct __align__(16) Shared {
   double uval[kMaxU];
   int ucol[kMaxU];
   double cupd[kMaxUpd];
+  double ccoef[kMaxUpd];  // coefficients in the working precision (update chain; Gram-Schmidt)
+  double cpart[kMaxThreads];  // partial sums of the update chain
+  long long cyc[16];
+  SolveCounts cnt;
   int alen, ulen;
   int iflag[12];
   int ilu_done, ilu_lost, ilu_flags, ilu_npiv;  // rows in flight (vmc_ilutp.cuh)
@@ -242,6 +259,22 @@ __device__ __forceinline__ bool task_solves(const Walker& w, const Params& P) {
   const int B = P.tri_group > 1 ? block_rows(w, P) : 0;
   return P.y_smem && !P.tri_sf && P.warp_rows == 0 && (P.tri_group <= 1 || (w.ex_col != nullptr && B >= 16)) &&
          w.n + B < 0xffff && (size_t)(w.n + B) * sizeof(T) <= (size_t)P.y_bytes && tasks_ahead<T>(P) >= 2;
+}
+
+// The walker's view into shared memory, for everything that runs on it.  Block-wide.
+__device__ __forceinline__ const Walker& stage_walker(Shared& sh, const Walker& view) {
+  static_assert(sizeof(Walker) % 8 == 0, "copied by 8-byte words");
+  __syncthreads();
+  const unsigned long long* src = reinterpret_cast<const unsigned long long*>(&view);
+  unsigned long long* dst = reinterpret_cast<unsigned long long*>(&sh.walk);
+  for (unsigned i = threadIdx.x; i < sizeof(Walker) / 8; i += blockDim.x) dst[i] = src[i];
+  __syncthreads();
+  return sh.walk;
+}
+__device__ __forceinline__ const Params& stage_params(Shared& sh, const Params& P) {
+  if (threadIdx.x == 0) sh.par = P;
+  __syncthreads();
+  return sh.par;
 }
 
 // ---- block-wide copies with several loads in flight per thread ---------------

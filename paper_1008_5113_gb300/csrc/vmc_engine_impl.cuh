@@ -38,12 +38,8 @@ __device__ __noinline__ void solve_with_controller(const Walker& w, const Params
   Ctl* c = w.ctl;
   const double rtol = P.inner_rtol;
   const int brow = w.row_of_part[k];
-  long long t0 = clock64();
-  solve_first<T>(w, P, brow, rtol, o, sh);
-  if (threadIdx.x == 0) c->cyc[PH_FIRST] += clock64() - t0;
-  t0 = clock64();
-  refine<T>(w, P, brow, rtol, 2 + P.max_restarts, o, sh);
-  if (threadIdx.x == 0) c->cyc[PH_REFINE] += clock64() - t0;
+  solve_move<T>(w, P, brow, rtol, 2 + P.max_restarts, o, sh);
+  flush_counts<T>(w, sh);
   if (o.status == ST_NOCONV && !c->fresh) {
     // out of cycles: reorder, refactor and solve again from scratch (Sec. 4)
     const int fl = factor_block<T>(w, P, sh, true);
@@ -55,11 +51,8 @@ __device__ __noinline__ void solve_with_controller(const Walker& w, const Params
       if (fl & 2) c->status = ST_CAPACITY;
     }
     __syncthreads();
-    const int brow2 = w.row_of_part[k];
-    t0 = clock64();
-    solve_first<T>(w, P, brow2, rtol, o, sh);
-    refine<T>(w, P, brow2, rtol, 4 * (2 + P.max_restarts), o, sh);  // and allow more cycles
-    if (threadIdx.x == 0) c->cyc[PH_REFINE] += clock64() - t0;
+    solve_move<T>(w, P, w.row_of_part[k], rtol, 4 * (2 + P.max_restarts), o, sh);  // and allow more cycles
+    flush_counts<T>(w, sh);
   }
   const int kits = o.its_trig >= 0 ? o.its_trig : o.total_its;  // iterations to the tolerance
   int cause = 0;
@@ -103,17 +96,29 @@ __device__ __noinline__ void solve_with_controller(const Walker& w, const Params
   __syncthreads();
 }
 
+// Entry t of particle k's row in the transposed copy.
+static __device__ __forceinline__ void store_ell(const Walker& w, int k, int t, int col, double val) {
+  const size_t at = ((size_t)(t >> 2) * w.ld + k) * 4 + (t & 3);
+  w.ell_col[at] = (unsigned short)col;
+  w.ell_val[at] = val;
+  if (w.ell_val32) w.ell_val32[at] = (float)val;
+}
+
 // Commit the move in shared memory for particle k (row replace + preconditioner update).
 template <typename T>
 __device__ __noinline__ void commit_move(const Walker& w, const Params& P, int k, double ratio, Shared& sh) {
   const int tid = threadIdx.x, nt = blockDim.x, n = w.n, cap = w.cap;
   const int alen = sh.alen, ulen = sh.ulen;
   const long long t0 = clock64();
+#pragma unroll 1
   for (int t = tid; t < alen; t += nt) {
     w.a_col[(size_t)k * cap + t] = sh.acol[t];
     w.a_val[(size_t)k * cap + t] = sh.aval[t];
-    w.a_val32[(size_t)k * cap + t] = (float)sh.aval[t];
+    if (w.a_val32) w.a_val32[(size_t)k * cap + t] = (float)sh.aval[t];
   }
+  if (w.ell_col)
+#pragma unroll 1
+    for (int t = tid; t < cap; t += nt) store_ell(w, k, t, t < alen ? sh.acol[t] : 0, t < alen ? sh.aval[t] : 0.0);
   if (tid == 0) {
     w.ctl->fresh = 0;
     w.a_len[k] = alen;
@@ -128,21 +133,37 @@ __device__ __noinline__ void commit_move(const Walker& w, const Params& P, int k
     T* Zh = (T*)w.upd_z;
     T* Uv = (T*)w.upd_uval;
     const double inv = 1.0 / ratio;
-    for (int i = tid; i < n; i += nt) Zh[(size_t)i * w.mu4 + s] = (T)(w.x64[i] * inv);  // transposed
-    for (int t = tid; t < ulen; t += nt) {
-      w.upd_ucol[(size_t)s * kMaxU + t] = sh.ucol[t];
-      Uv[(size_t)s * kMaxU + t] = (T)sh.uval[t];
+    T* zs = Zh + (size_t)s * w.ld;
+#pragma unroll 1
+    for (int i = tid; i < n; i += nt) zs[i] = (T)(w.x64[i] * inv);
+#pragma unroll 1
+    for (int t = tid; t < ulen; t += nt) {  // the update index fastest: see update_chain
+      w.upd_ucol[(size_t)t * kMaxUpd + s] = sh.ucol[t];
+      Uv[(size_t)t * kMaxUpd + s] = (T)sh.uval[t];
     }
     if (tid == 0) { w.upd_ulen[s] = ulen; c->upd_nnz += ulen; }
     __syncthreads();
-    // G[s][t] = u_s^T z_hat_t for t < s, from the stored (working-precision) values
+    // g_t = u_s^T z_hat_t for t < s, from the stored (working-precision) values, and row s of
+    // the inverse of the unit lower matrix I + G: -g_t - sum_{t < q < s} g_q (inverse)_qt.
+    // (A trailing block of the inverse is the inverse of the trailing block: dropping the
+    // oldest updates drops its first rows and columns.)
     const int lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
+#pragma unroll 1
     for (int t = wid; t < s; t += nw) {
       double acc = 0.0;
+#pragma unroll 1
       for (int e = lane; e < ulen; e += 32)
-        acc += (double)Uv[(size_t)s * kMaxU + e] * (double)Zh[(size_t)w.upd_ucol[(size_t)s * kMaxU + e] * w.mu4 + t];
+        acc += (double)(T)sh.uval[e] * (double)Zh[(size_t)t * w.ld + sh.ucol[e]];
       acc = warp_sum(acc);
-      if (lane == 0) w.upd_G[(size_t)s * kMaxUpd + t] = acc;
+      if (lane == 0) sh.cupd[t] = acc;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int t = tid; t < s; t += nt) {
+      double acc = sh.cupd[t];
+#pragma unroll 4
+      for (int q = t + 1; q < s; ++q) acc += sh.cupd[q] * w.upd_G[(size_t)t * kMaxUpd + q];
+      w.upd_G[(size_t)t * kMaxUpd + s] = -acc;  // column s of the transpose
     }
     __syncthreads();
     if (tid == 0) c->n_upd = s + 1;
@@ -199,7 +220,7 @@ __device__ __noinline__ void mc_step(const Walker& w, const Params& P, int k, ui
   }
   __syncthreads();
   if (!build_move(w, k, sh)) return;
-  if (threadIdx.x == 0) c->cyc[PH_BUILD] += clock64() - t_step;
+  if (threadIdx.x == 0) sh.cyc[PH_BUILD] += clock64() - t_step;
   SolveOut o;
   solve_with_controller<T>(w, P, k, o, sh);
   const double U = accept_uniform(seed, sweep, (uint32_t)k);
@@ -243,7 +264,8 @@ static __device__ void af_take_stats(Ctl* c, Ctl* sc) {
 }
 
 // Block-wide: adopt factor set af_target and keep the chain entries s0 .. n_upd - 1
-// (moved to 0 .. n_upd - 1 - s0; G[s][t] = u_s^T z_hat_t does not depend on the root).
+// (moved to 0 .. n_upd - 1 - s0; G[s][t] = u_s^T z_hat_t does not depend on the root, and
+// the inverse of I + G restricts to the kept entries).
 template <typename T>
 __device__ void af_swap(const Walker& w0, const Params& P, Shared& sh) {
   Ctl* c = w0.ctl;
@@ -251,25 +273,39 @@ __device__ void af_swap(const Walker& w0, const Params& P, Shared& sh) {
   const int tid = threadIdx.x, nt = blockDim.x, n = w0.n;
   const int s0 = c->af_snap, len = c->n_upd - s0;
   T* Zt = (T*)w0.upd_z;
-  const int mcap = w0.mu4;
-  for (int i = tid; i < n; i += nt) {
-    T* zr = Zt + (size_t)i * mcap;
-    for (int j = 0; j < len; ++j) zr[j] = zr[s0 + j];
-  }
+#pragma unroll 1
+  for (int i = tid; i < n; i += nt)
+#pragma unroll 8
+    for (int j = 0; j < len; ++j) Zt[(size_t)j * w0.ld + i] = Zt[(size_t)(s0 + j) * w0.ld + i];
+  // the kept updates move down by s0; every thread moves rows of its own, in increasing order
   T* Uv = (T*)w0.upd_uval;
-  for (int j = 0; j < len; ++j) {  // destination rows in increasing order: sources are intact
-    const int ul = w0.upd_ulen[s0 + j];
-    for (int t = tid; t < ul; t += nt) {
-      w0.upd_ucol[(size_t)j * kMaxU + t] = w0.upd_ucol[(size_t)(s0 + j) * kMaxU + t];
-      Uv[(size_t)j * kMaxU + t] = Uv[(size_t)(s0 + j) * kMaxU + t];
-    }
-    for (int t = tid; t < j; t += nt) w0.upd_G[(size_t)j * kMaxUpd + t] = w0.upd_G[(size_t)(s0 + j) * kMaxUpd + s0 + t];
-    __syncthreads();
-    if (tid == 0) w0.upd_ulen[j] = ul;
+#pragma unroll 1
+  for (int t = tid; t < kMaxU; t += nt) {
+    int* uc = w0.upd_ucol + (size_t)t * kMaxUpd;
+    T* uu = Uv + (size_t)t * kMaxUpd;
+#pragma unroll 1
+    for (int j = 0; j < len; ++j)
+      if (t < w0.upd_ulen[s0 + j]) {
+        uc[j] = uc[s0 + j];
+        uu[j] = uu[s0 + j];
+      }
   }
+  __syncthreads();
+  double* Gi = w0.upd_G;
+#pragma unroll 1
+  for (int t0 = 0; t0 < len; ++t0) {  // row t0 of the transposed inverse from row s0 + t0
+#pragma unroll 1
+    for (int j = t0 + 1 + tid; j < len; j += nt) Gi[(size_t)t0 * kMaxUpd + j] = Gi[(size_t)(s0 + t0) * kMaxUpd + s0 + j];
+    __syncthreads();
+  }
+  int ul = 0;
+  if (tid < len) ul = w0.upd_ulen[s0 + tid];
+  __syncthreads();
+  if (tid < len) w0.upd_ulen[tid] = ul;
   if (P.af_reorder) {
     // the new row pairing comes with the factors; the chain lives in column space and
     // x = A_p^{-1} e_{row(k)} does not depend on the row order, so it carries over
+#pragma unroll 1
     for (int r = tid; r < n; r += nt) {
       w0.part_of_row[r] = w0.snap_part[r];
       w0.row_of_part[r] = w0.snap_rop[r];
@@ -278,6 +314,7 @@ __device__ void af_swap(const Walker& w0, const Params& P, Shared& sh) {
   __syncthreads();
   if (tid == 0) {
     int nnzu = 0;
+#pragma unroll 1
     for (int j = 0; j < len; ++j) nnzu += w0.upd_ulen[j];
     c->upd_nnz = nnzu;
     c->n_upd = len;
@@ -340,6 +377,7 @@ __device__ __noinline__ void af_step_begin(const Walker& w0, const Params& P, Sh
   if (act == 1) {
     fence_acq_rel_gpu();
     af_swap<T>(w0, P, sh);
+    stage_walker(sh, active_of(w0));
   } else if (act == 2) {
     const int fl = factor_block<T>(active_of(w0), P, sh, true);
     if (threadIdx.x == 0) {
@@ -354,15 +392,18 @@ __device__ __noinline__ void af_step_begin(const Walker& w0, const Params& P, Sh
   __syncthreads();
   if (sh.iflag[7]) {
     const int n = w0.n, tid = threadIdx.x, nt = blockDim.x;
+#pragma unroll 1
     for (size_t idx = tid; idx < (size_t)n * w0.cap; idx += nt) {
       w0.snap_col[idx] = w0.a_col[idx];
       w0.snap_val[idx] = w0.a_val[idx];
     }
+#pragma unroll 1
     for (int p = tid; p < n; p += nt) {
       w0.snap_len[p] = w0.a_len[p];
       w0.snap_part[p] = w0.part_of_row[p];
     }
     if (P.af_reorder)
+#pragma unroll 1
       for (int i = tid; i < 3 * n; i += nt) w0.snap_R[i] = w0.R[i];
     __syncthreads();
     if (tid == 0) {
@@ -406,7 +447,7 @@ __device__ __noinline__ void af_factor_loop(const Walker& w0, const Params& P, i
     __syncthreads();
     if (sh.iflag[5] != 1) break;  // the solver's own bounded waits report a lost partner
     fence_acq_rel_gpu();
-    const Walker& wf = *w0.fact[sh.iflag[6]];
+    const Walker& wf = stage_walker(sh, *w0.fact[sh.iflag[6]]);
     const int fl = factor_block<T>(wf, P, sh, P.af_reorder != 0);
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -441,7 +482,7 @@ __device__ void advance_budget(const Walker& w0, const Params& P, long long swee
     __syncthreads();
     if (!go) break;
     if (PAIR) af_step_begin<T>(w0, P, sh);
-    mc_step<T>(active_of(w0), P, k, seed, (uint32_t)sw, sigma, nullptr, nullptr, sh);
+    mc_step<T>(sh.walk, P, k, seed, (uint32_t)sw, sigma, nullptr, nullptr, sh);
     if (++k == lim) { k = 0; ++sw; }
   }
   if (threadIdx.x == 0) { c->pos_sweep = sw; c->pos_k = k; c->pos_valid = 1; }
@@ -450,21 +491,24 @@ __device__ void advance_budget(const Walker& w0, const Params& P, long long swee
 // ---------------------------------------------------------------------------
 // kernels
 // ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(kMaxThreads, 2) k_sweep(const Walker* __restrict__ W, int walker0, Params P, int n_sweeps,
+template <typename T, int kPerSm>
+__global__ void __launch_bounds__(kMaxThreads, kPerSm) k_sweep(const Walker* __restrict__ W, int walker0, Params P_, int n_sweeps,
                                                 long long sweep0, double sigma, const uint64_t* __restrict__ seeds,
                                                 uint8_t* acc_log, double* ratio_log) {
   __shared__ Shared sh;
+  const Params& P = stage_params(sh, P_);
   ring_init(sh, P);
   const int wi = walker0 + blockIdx.x;
-  const Walker& w = active_of(W[wi]);
+  const Walker& w = stage_walker(sh, active_of(W[wi]));
   const uint64_t seed = seeds[wi];
   const int n = w.n;
   if (P.budget_ctr) {
-    advance_budget<T, false>(W[wi], P, sweep0, sigma, seed, sh);
+    advance_budget<T, false>(w, P, sweep0, sigma, seed, sh);
     return;
   }
+#pragma unroll 1
   for (int s = 0; s < n_sweeps; ++s)
+#pragma unroll 1
     for (int k = 0; k < (P.step_limit > 0 ? min(n, P.step_limit) : n); ++k) {
       const long long idx = (long long)n_sweeps * w.log_base + (long long)s * n + k;
       mc_step<T>(w, P, k, seed, (uint32_t)(sweep0 + s), sigma, acc_log ? acc_log + idx : nullptr,
@@ -477,11 +521,12 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_sweep(const Walker* __restri
 // rank 0 steps (as k_sweep), rank 1 factors (af_factor_loop).  launch_id: unique per
 // launch of this context, > 0.
 template <typename T>
-__global__ void __launch_bounds__(kMaxThreads, 2) k_sweep_pair(const Walker* __restrict__ W, int walker0, Params P,
+__global__ void __launch_bounds__(kMaxThreads, 1) k_sweep_pair(const Walker* __restrict__ W, int walker0, Params P_,
                                                      int n_sweeps, long long sweep0, double sigma,
                                                      const uint64_t* __restrict__ seeds, uint8_t* acc_log,
                                                      double* ratio_log, int launch_id) {
   __shared__ Shared sh;
+  const Params& P = stage_params(sh, P_);
   ring_init(sh, P);
   const int wi = walker0 + (int)(blockIdx.x >> 1);
   const Walker& w0 = W[wi];
@@ -491,13 +536,16 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_sweep_pair(const Walker* __r
   }
   const uint64_t seed = seeds[wi];
   const int n = w0.n;
+  stage_walker(sh, active_of(w0));
   if (P.budget_ctr) {
     advance_budget<T, true>(w0, P, sweep0, sigma, seed, sh);
   } else {
+#pragma unroll 1
     for (int s = 0; s < n_sweeps; ++s)
+#pragma unroll 1
       for (int k = 0; k < (P.step_limit > 0 ? min(n, P.step_limit) : n); ++k) {
         af_step_begin<T>(w0, P, sh);
-        const Walker& w = active_of(w0);
+        const Walker& w = sh.walk;  // the active view
         const long long idx = (long long)n_sweeps * w.log_base + (long long)s * n + k;
         mc_step<T>(w, P, k, seed, (uint32_t)(sweep0 + s), sigma, acc_log ? acc_log + idx : nullptr,
                    ratio_log ? ratio_log + idx : nullptr, sh);
@@ -508,16 +556,17 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_sweep_pair(const Walker* __r
 }
 
 // One step (particle q of sweep s_local of a batch of n_sweeps) for every walker in the grid.
-template <typename T>
-__global__ void __launch_bounds__(kMaxThreads, 2) k_step(const Walker* __restrict__ W, int walker0, Params P, int q, int n_sweeps,
+template <typename T, int kPerSm>
+__global__ void __launch_bounds__(kMaxThreads, kPerSm) k_step(const Walker* __restrict__ W, int walker0, Params P_, int q, int n_sweeps,
                                                int s_local, long long sweep0, double sigma,
                                                const uint64_t* __restrict__ seeds, uint8_t* acc_log, double* ratio_log,
                                                const long long* __restrict__ sweep_dev) {
   __shared__ Shared sh;
   const int wi = walker0 + blockIdx.x;
-  const Walker& w = active_of(W[wi]);
-  if (q >= w.n) return;
+  if (q >= W[wi].n) return;
+  const Params& P = stage_params(sh, P_);
   ring_init(sh, P);
+  const Walker& w = stage_walker(sh, active_of(W[wi]));
   if (sweep_dev) sweep0 = *sweep_dev;  // graph replays: the sweep index lives on the device
   const long long idx = (long long)n_sweeps * w.log_base + (long long)s_local * w.n + q;
   mc_step<T>(w, P, q, seeds[wi], (uint32_t)(sweep0 + s_local), sigma, acc_log ? acc_log + idx : nullptr,
@@ -526,11 +575,12 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_step(const Walker* __restric
 
 // Single-move API: ratio for particle k moved to r_new (no commit); result in ctl.
 template <typename T>
-__global__ void __launch_bounds__(kMaxThreads, 2) k_ratio(const Walker* __restrict__ W, int wi, Params P, int k, double rx,
+__global__ void __launch_bounds__(kMaxThreads, 1) k_ratio(const Walker* __restrict__ W, int wi, Params P_, int k, double rx,
                                                 double ry, double rz, int want_grad) {
   __shared__ Shared sh;
+  const Params& P = stage_params(sh, P_);
   ring_init(sh, P);
-  const Walker& w = active_of(W[wi]);
+  const Walker& w = stage_walker(sh, active_of(W[wi]));
   Ctl* c = w.ctl;
   if (threadIdx.x == 0) {
     sh.rnew[0] = wrap_box(rx, w.L);
@@ -547,6 +597,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_ratio(const Walker* __restri
     // grad ln|det A'| = sum_o grad phi_o(r') z_o / ratio with grad phi = -2 kappa (r' - Z_o) phi,
     // lap det A' / det A' = sum_o (4 kappa^2 d^2 - 6 kappa) phi z_o / ratio
     double g[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
     for (int t = threadIdx.x; t < sh.alen; t += blockDim.x) {
       const int col = sh.acol[t];
       const double* zo = w.Z + 3 * w.orb_of_col[col];
@@ -559,13 +610,16 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_ratio(const Walker* __restri
       g[2] += -2.0 * w.kappa * dz * pz;
       g[3] += (4.0 * w.kappa * w.kappa * (dx * dx + dy * dy + dz * dz) - 6.0 * w.kappa) * pz;
     }
+#pragma unroll 1
     for (int d = 0; d < 4; ++d) g[d] = block_sum(g[d], sh);
     if (threadIdx.x == 0) {
       for (int d = 0; d < 3; ++d) c->pend_grad[d] = g[d] / o.ratio;
       c->pend_lap = g[3] / o.ratio;
     }
   }
+#pragma unroll 1
   for (int t = threadIdx.x; t < sh.alen; t += blockDim.x) { w.pend_acol[t] = sh.acol[t]; w.pend_aval[t] = sh.aval[t]; }
+#pragma unroll 1
   for (int t = threadIdx.x; t < sh.ulen; t += blockDim.x) { w.pend_ucol[t] = sh.ucol[t]; w.pend_uval[t] = sh.uval[t]; }
   if (threadIdx.x == 0) {
     c->pend_alen = sh.alen;
@@ -579,10 +633,11 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_ratio(const Walker* __restri
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kMaxThreads, 2) k_accept(const Walker* __restrict__ W, int wi, Params P) {
+__global__ void __launch_bounds__(kMaxThreads, 1) k_accept(const Walker* __restrict__ W, int wi, Params P_) {
   __shared__ Shared sh;
+  const Params& P = stage_params(sh, P_);
   ring_init(sh, P);
-  const Walker& w = active_of(W[wi]);
+  const Walker& w = stage_walker(sh, active_of(W[wi]));
   Ctl* c = w.ctl;
   const int valid = c->pend_valid;
   const int k = c->pend_k;
@@ -592,7 +647,9 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_accept(const Walker* __restr
     sh.rnew[0] = c->pend_r[0]; sh.rnew[1] = c->pend_r[1]; sh.rnew[2] = c->pend_r[2];
   }
   __syncthreads();
+#pragma unroll 1
   for (int t = threadIdx.x; t < sh.alen; t += blockDim.x) { sh.acol[t] = w.pend_acol[t]; sh.aval[t] = w.pend_aval[t]; }
+#pragma unroll 1
   for (int t = threadIdx.x; t < sh.ulen; t += blockDim.x) { sh.ucol[t] = w.pend_ucol[t]; sh.uval[t] = w.pend_uval[t]; }
   __syncthreads();
   commit_move<T>(w, P, k, c->pend_ratio, sh);
@@ -604,18 +661,21 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_accept(const Walker* __restr
 // of A^{-1}, indexed by orbital), contracted with the particle's own Slater row weighted by
 // the Laplacian factor of each Gaussian; the weighted row takes the place of u, so the FP64
 // refinement controls the error of this contraction.  One CTA per walker; out[walker].
-template <typename T>
-__global__ void __launch_bounds__(kMaxThreads, 2) k_kinetic(const Walker* __restrict__ W, Params P, double* out) {
+template <typename T, int kPerSm>
+__global__ void __launch_bounds__(kMaxThreads, kPerSm) k_kinetic(const Walker* __restrict__ W, Params P_, double* out) {
   __shared__ Shared sh;
+  const Params& P = stage_params(sh, P_);
   ring_init(sh, P);
-  const Walker& w = active_of(W[blockIdx.x]);
+  const Walker& w = stage_walker(sh, active_of(W[blockIdx.x]));
   const int n = w.n, cap = w.cap;
   const double kap = w.kappa;
   double e = 0.0;
+#pragma unroll 1
   for (int k = 0; k < n; ++k) {
     if (w.ctl->status != ST_OK) break;  // read by every thread after the last barrier
     const int len = w.a_len[k];
     const double rk[3] = {w.R[3 * k], w.R[3 * k + 1], w.R[3 * k + 2]};
+#pragma unroll 1
     for (int t = threadIdx.x; t < len; t += blockDim.x) {
       const int col = w.a_col[(size_t)k * cap + t];
       const double d2 = dist2(rk, w.Z + 3 * w.orb_of_col[col], w.L);
@@ -635,13 +695,15 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_kinetic(const Walker* __rest
 // All Slater rows from the positions (warp per particle), then the initial pairing
 // (particle i with orbital i), the greedy reordering and the first factorisation.
 template <typename T>
-__global__ void __launch_bounds__(kMaxThreads, 2) k_setup(const Walker* __restrict__ W, int walker0, Params P) {
+__global__ void __launch_bounds__(kMaxThreads, 1) k_setup(const Walker* __restrict__ W, int walker0, Params P_) {
   __shared__ Shared sh;
+  const Params& P = stage_params(sh, P_);
   ring_init(sh, P);
-  const Walker& w = active_of(W[walker0 + blockIdx.x]);
+  const Walker& w = stage_walker(sh, active_of(W[walker0 + blockIdx.x]));
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   Ctl* c = w.ctl;
   int bad = 0;
+#pragma unroll 1
   for (int p = wid; p < w.n; p += nw) {
     const int len = build_row_warp(w, w.R + 3 * p, w.a_col + (size_t)p * w.cap, w.a_val + (size_t)p * w.cap, w.cap);
     if (lane == 0) {
@@ -650,7 +712,18 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_setup(const Walker* __restri
     }
   }
   __syncthreads();
-  for (int idx = threadIdx.x; idx < w.n * w.cap; idx += blockDim.x) w.a_val32[idx] = (float)w.a_val[idx];
+  if (w.a_val32)
+#pragma unroll 1
+    for (int idx = threadIdx.x; idx < w.n * w.cap; idx += blockDim.x) w.a_val32[idx] = (float)w.a_val[idx];
+  if (w.ell_col)
+#pragma unroll 1
+    for (int t = 0; t < w.cap; ++t)
+#pragma unroll 1
+      for (int p = threadIdx.x; p < w.n; p += blockDim.x) {
+        const bool in = t < w.a_len[p];
+        store_ell(w, p, t, in ? w.a_col[(size_t)p * w.cap + t] : 0, in ? w.a_val[(size_t)p * w.cap + t] : 0.0);
+      }
+#pragma unroll 1
   for (int col = threadIdx.x; col < w.n; col += blockDim.x) {
     const int o = w.orb_of_col[col];
     w.part_of_row[col] = o;
@@ -670,57 +743,73 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_setup(const Walker* __restri
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kMaxThreads, 2) k_refactor(const Walker* __restrict__ W, int wi, Params P, int reorder) {
+__global__ void __launch_bounds__(kMaxThreads, 1) k_refactor(const Walker* __restrict__ W, int wi, Params P_, int reorder) {
   __shared__ Shared sh;
+  const Params& P = stage_params(sh, P_);
   ring_init(sh, P);
-  const Walker& w = active_of(W[wi]);
+  const Walker& w = stage_walker(sh, active_of(W[wi]));
   factor_block<T>(w, P, sh, reorder != 0);
   if (threadIdx.x == 0 && sh.iflag[3]) w.ctl->status = ST_TIMEOUT;
 }
 
 // z = M v for the test entry point: v in r64 (FP64), result in x64 (FP64).
 template <typename T>
-__global__ void __launch_bounds__(kMaxThreads, 2) k_apply_precond(const Walker* __restrict__ W, int wi, Params P) {
+__global__ void __launch_bounds__(kMaxThreads, 1) k_apply_precond(const Walker* __restrict__ W, int wi, Params P_) {
   __shared__ Shared sh;
-  const Walker& w = active_of(W[wi]);
+  const Params& P = stage_params(sh, P_);
+  const Walker& w = stage_walker(sh, active_of(W[wi]));
   ring_init(sh, P);
   T* V = (T*)w.V;
   T* Zk = (T*)w.Zk;
+#pragma unroll 1
   for (int i = threadIdx.x; i < w.n; i += blockDim.x) V[i] = (T)w.r64[i];
   __syncthreads();
-  precond_apply<T>(w, P, V, Zk, sh);
+  precond_apply<T, false>(w, P, V, Zk, sh);
+#pragma unroll 1
   for (int i = threadIdx.x; i < w.n; i += blockDim.x) w.x64[i] = (double)Zk[i];
+  flush_counts<T>(w, sh);
 }
 
 // Microbenchmark: `reps` back-to-back applications of one hot-path kernel per walker
 // (0: L and U triangular solves, 1: SpMV in the working precision, 2: the full
 // preconditioner apply with the update chain), on V[0] = 1 / sqrt(n).
 template <typename T>
-__global__ void __launch_bounds__(kMaxThreads, 2) k_bench(const Walker* __restrict__ W, Params P, int which, int reps) {
+__global__ void __launch_bounds__(kMaxThreads, 2) k_bench(const Walker* __restrict__ W, Params P_, int which, int reps) {
   __shared__ Shared sh;
+  const Params& P = stage_params(sh, P_);
   ring_init(sh, P);
-  const Walker& w = active_of(W[blockIdx.x]);
+  const Walker& w = stage_walker(sh, active_of(W[blockIdx.x]));
   const int n = w.n;
   T* V = (T*)w.V;
   T* Zk = (T*)w.Zk;
+#pragma unroll 1
   for (int i = threadIdx.x; i < n; i += blockDim.x) V[i] = (T)rsqrt((double)n);
   __syncthreads();
+  const bool sm = krylov_in_smem<T>(w, P);
+#pragma unroll 1
   for (int it = 0; it < reps; ++it) {
     if (which == 0) {
       const long long t0 = clock64();
       const T* y = tri_both<T>(w, P, V, sh);
-      if (threadIdx.x == 0) w.ctl->cyc[PH_TRI] += clock64() - t0;
+      if (threadIdx.x == 0) sh.cyc[PH_TRI] += clock64() - t0;
       block_scatter(Zk, w.perm, y, n);
       if (threadIdx.x == 0)
         w.ctl->alg_bytes += w.ctl->nnz_LU * (sizeof(T) + 4) + (double)n * (3 * sizeof(T) + 8);
     } else if (which == 1) {
-      spmv<T>(w, P, stage_x<T>(w, P, V), Zk);
+      if (sm) {  // as in an iteration: the input in the task ring, the result in the solve area
+        block_copy(z_ring<T>(P), V, n);
+        __syncthreads();
+        spmv<T>(w, z_ring<T>(P), (const T*)nullptr, (T*)dyn_smem());
+      } else {
+        spmv<T>(w, V, (const T*)nullptr, Zk);
+      }
       if (threadIdx.x == 0) w.ctl->alg_bytes += w.ctl->nnz_A * (sizeof(T) + 4) + (double)n * (2 * sizeof(T) + 4);
     } else {
-      precond_apply<T>(w, P, V, Zk, sh);
+      precond_apply<T, false>(w, P, V, Zk, sh);
     }
     __syncthreads();
   }
+  flush_counts<T>(w, sh);
 }
 
 
@@ -740,16 +829,23 @@ static cudaError_t prep(K kernel, const LaunchCfg& L) {
     return cudaGetLastError();                                         \
   } while (0)
 
+// The sweeping kernels exist for one and for two CTAs an SM (255 and 128 registers a thread).
+#define VMC_LAUNCH_PER_SM(KERNEL, GRID, ...)                         \
+  do {                                                               \
+    if (L.per_sm > 1) VMC_LAUNCH((KERNEL<T, 2>), GRID, __VA_ARGS__); \
+    VMC_LAUNCH((KERNEL<T, 1>), GRID, __VA_ARGS__);                   \
+  } while (0)
+
 template <typename T>
 int kernel_static_smem_T() {
   cudaFuncAttributes a{};
-  cudaFuncGetAttributes(&a, k_sweep<T>);
+  cudaFuncGetAttributes(&a, k_accept<T>);
   return (int)a.sharedSizeBytes;
 }
 template <typename T>
 cudaError_t launch_sweep_T(const LaunchCfg& L, const Walker* W, int walker0, int nwalk, const Params& P, int n_sweeps,
                            long long sweep0, double sigma, const uint64_t* seeds, uint8_t* acc, double* ratio) {
-  VMC_LAUNCH(k_sweep<T>, nwalk, W, walker0, P, n_sweeps, sweep0, sigma, seeds, acc, ratio);
+  VMC_LAUNCH_PER_SM(k_sweep, nwalk, W, walker0, P, n_sweeps, sweep0, sigma, seeds, acc, ratio);
 }
 template <typename T>
 cudaError_t launch_sweep_pair_T(const LaunchCfg& L, const Walker* W, int walker0, int nwalk, const Params& P,
@@ -772,12 +868,12 @@ cudaError_t launch_sweep_pair_T(const LaunchCfg& L, const Walker* W, int walker0
   return cudaLaunchKernelEx(&lc, k_sweep_pair<T>, W, walker0, P, n_sweeps, sweep0, sigma, seeds, acc, ratio, launch_id);
 }
 template <typename T>
-cudaError_t prepare_step_kernels_T(const LaunchCfg& L) { return prep(k_step<T>, L); }
+cudaError_t prepare_step_kernels_T(const LaunchCfg& L) { return L.per_sm > 1 ? prep(k_step<T, 2>, L) : prep(k_step<T, 1>, L); }
 template <typename T>
 cudaError_t launch_step_T(const LaunchCfg& L, const Walker* W, int walker0, int nwalk, const Params& P, int q,
                           int n_sweeps, int s_local, long long sweep0, double sigma, const uint64_t* seeds,
                           uint8_t* acc, double* ratio, const long long* sweep_dev) {
-  VMC_LAUNCH(k_step<T>, nwalk, W, walker0, P, q, n_sweeps, s_local, sweep0, sigma, seeds, acc, ratio, sweep_dev);
+  VMC_LAUNCH_PER_SM(k_step, nwalk, W, walker0, P, q, n_sweeps, s_local, sweep0, sigma, seeds, acc, ratio, sweep_dev);
 }
 template <typename T>
 cudaError_t launch_ratio_T(const LaunchCfg& L, const Walker* W, int wi, const Params& P, int k, const double r[3],
@@ -786,7 +882,7 @@ cudaError_t launch_ratio_T(const LaunchCfg& L, const Walker* W, int wi, const Pa
 }
 template <typename T>
 cudaError_t launch_kinetic_T(const LaunchCfg& L, const Walker* W, int nwalk, const Params& P, double* out) {
-  VMC_LAUNCH(k_kinetic<T>, nwalk, W, P, out);
+  VMC_LAUNCH_PER_SM(k_kinetic, nwalk, W, P, out);
 }
 template <typename T>
 cudaError_t launch_accept_T(const LaunchCfg& L, const Walker* W, int wi, const Params& P) {

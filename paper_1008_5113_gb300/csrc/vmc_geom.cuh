@@ -122,6 +122,7 @@ __device__ __forceinline__ int build_row_warp(const Walker& w, const double* r, 
   const int lane = threadIdx.x & 31;
   const CandBox b = cand_box(w, r);
   int cnt = 0;
+#pragma unroll 1
   for (int base = 0; base < b.total; base += 32) {
     const int q = base + lane;
     bool keep = false;
@@ -155,6 +156,7 @@ __device__ __forceinline__ int build_u_warp(const Walker& w, int p, const int* a
   const int* oc = w.a_col + (size_t)p * w.cap;
   const double* ov = w.a_val + (size_t)p * w.cap;
   int cnt = 0;
+#pragma unroll 1
   for (int base = 0; base < alen; base += 32) {
     const int t = base + lane;
     double v = 0.0;
@@ -162,6 +164,7 @@ __device__ __forceinline__ int build_u_warp(const Walker& w, int p, const int* a
     if (t < alen) {
       c = acol[t];
       v = aval[t];
+#pragma unroll 1
       for (int s = 0; s < olen; ++s)
         if (oc[s] == c) { v = __dsub_rn(v, ov[s]); break; }
     }
@@ -169,6 +172,7 @@ __device__ __forceinline__ int build_u_warp(const Walker& w, int p, const int* a
     if (t < alen) { ucol[cnt + t - base] = c; uval[cnt + t - base] = v; }
     cnt += __popc(m);
   }
+#pragma unroll 1
   for (int base = 0; base < olen; base += 32) {
     const int t = base + lane;
     bool extra = false;
@@ -177,6 +181,7 @@ __device__ __forceinline__ int build_u_warp(const Walker& w, int p, const int* a
     if (t < olen) {
       c = oc[t];
       extra = true;
+#pragma unroll 1
       for (int s = 0; s < alen; ++s)
         if (acol[s] == c) { extra = false; break; }
       v = -ov[t];

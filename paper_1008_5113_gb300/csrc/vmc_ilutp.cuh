@@ -70,6 +70,7 @@ __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared&
   unsigned short* ip = (unsigned short*)(dsm + pl.o_ip);
   volatile int* done = &sh.ilu_done;
   volatile int* lost = &sh.ilu_lost;
+#pragma unroll 1
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     perm[i] = (unsigned short)i;
     ip[i] = (unsigned short)i;
@@ -85,6 +86,7 @@ __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared&
   int p = P.lfil_extra;
   if (p < 0) {
     long long tot = 0;
+#pragma unroll 1
     for (int i = lane; i < n; i += 32) tot += w.a_len[i];
     tot = warp_sum_ll(tot);
     p = (int)((tot + 2LL * n - 1) / (2LL * n));  // ceil(avg nnz per row / 2)
@@ -106,8 +108,11 @@ __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared&
     unsigned short* bnd = (unsigned short*)(mine + pl.o_bnd);
     auto at = [&](int s) -> W& { return s < kPipeVals ? val[s] : over[s]; };
     const int nwords = (n + 31) >> 5, nsum = (nwords + 31) >> 5;
+#pragma unroll 1
     for (int i = lane; i < nwords; i += 32) lbits[i] = 0u;
+#pragma unroll 1
     for (int i = lane; i < nsum; i += 32) lsum[i] = 0u;
+#pragma unroll 1
     for (int i = lane; i < n; i += 32) wpos[i] = 0xffffu;
     __syncwarp();
     auto mark = [&](int f) {
@@ -116,6 +121,7 @@ __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared&
     };
     int flags = 0, npiv = 0;
     long long n_elim = 0, n_cand = 0, nnz = 0;
+#pragma unroll 1
     for (int r = wid; r < n; r += NW) {
       const int part = w.part_of_row[r];
       const int len = w.a_len[part];
@@ -124,6 +130,7 @@ __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared&
       int d = __shfl_sync(0xffffffffu, *done, 0);  // labels below d are final
       __threadfence_block();
       double ss = 0.0;
+#pragma unroll 1
       for (int t = lane; t < len; t += 32) {
         const int c = ac[t];
         const double v = av[t];
@@ -151,6 +158,7 @@ __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared&
             best = (w0 << 5) + __ffs(cur) - 1;
           } else {
             const int s0 = (w0 + 1) >> 5;  // summary word holding bitmap word w0 + 1
+#pragma unroll 1
             for (int sb = s0; sb < nsum && best == 0x7fffffff; sb += 32) {
               const int si = sb + lane;
               unsigned sv = si < nsum ? lsum[si] : 0u;
@@ -181,6 +189,7 @@ __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared&
           if (d2 == d) break;  // gave up
           __threadfence_block();
           d2 = min(d2, r);
+#pragma unroll 1
           for (int k = d + lane; k < d2; k += 32)
             if (wpos[perm[k]] != 0xffffu) mark(k);
           d = d2;
@@ -203,6 +212,7 @@ __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared&
           continue;
         }
         if (lane == 0) at(tb) = wk;
+#pragma unroll 1
         for (int base = 0; base < ul; base += 32) {
           const int t = base + lane;
           const bool valid = t < ul;
@@ -237,6 +247,7 @@ __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared&
       n_cand += cnt;
       // entries of the original row on either side (labels below r are final now)
       int nl = 0, nu = 0;
+#pragma unroll 1
       for (int t = lane; t < len; t += 32) {
         const int f = ip[nz[t]];
         nl += f < r;
@@ -247,6 +258,7 @@ __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared&
       // candidates on one side: L keeps every nonzero multiplier, U the entries above threshold
       auto compact = [&](bool upper) {
         int c = 0;
+#pragma unroll 1
         for (int base = 0; base < cnt; base += 32) {
           const int t = base + lane;
           bool k = false;
@@ -273,6 +285,7 @@ __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared&
       select_topk<K>(hist, bnd, selk, cU, nu + pk, key, label);
       K bk = 0;
       int bf = 0x7fffffff, be = 0;
+#pragma unroll 1
       for (int e = lane; e < cU; e += 32)
         if (selk[e]) {
           const K m = key(e);
@@ -304,6 +317,7 @@ __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared&
         ++npiv;
       }
       int nU = 0;
+#pragma unroll 1
       for (int base = 0; base < cU; base += 32) {
         const int e = base + lane;
         bool k = e < cU && selk[e];
@@ -340,6 +354,7 @@ __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared&
       const int cL = compact(false);
       select_topk<K>(hist, bnd, selk, cL, nl + pk, key, label);
       int nL = 0;
+#pragma unroll 1
       for (int base = 0; base < cL; base += 32) {
         const int e = base + lane;
         const bool k = e < cL && selk[e];
@@ -355,6 +370,7 @@ __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared&
       if (lane == 0) w.l_len[r] = nL;
       nnz += nL + nU + 1;
       // clear the working row (and the pending-label bitmaps)
+#pragma unroll 1
       for (int t = lane; t < cnt; t += 32) {
         const int c = nz[t];
         const int f = ip[c];
@@ -372,6 +388,7 @@ __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared&
     }
   }
   __syncthreads();
+#pragma unroll 1
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     w.perm[i] = perm[i];
     w.iperm[i] = ip[i];

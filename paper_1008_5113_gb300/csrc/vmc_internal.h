@@ -15,6 +15,7 @@ struct LaunchCfg {
   int threads;
   bool fp64;
   size_t smem;  // dynamic shared memory per walker CTA
+  int per_sm;   // walker CTAs an SM is to hold (1 or 2)
 };
 // static shared memory of the walker kernels (bytes)
 int kernel_static_smem(bool fp64);

@@ -153,10 +153,11 @@ extern "C" vmc_status vmc_ratio_noalloc(const vmc_system* sys, const vmc_solver_
   const size_t oLlp = o.take<int>(n + 1), oLlr = o.take<int>(n), oUlp = o.take<int>(n + 1), oUlr = o.take<int>(n);
   const size_t oCur = o.take<int>(n + 1), oWr = o.take<double>(n), oWp = o.take<int>(n);
   const size_t oGP = o.take<int>(n), oGQ = o.take<int>(n);
-  const size_t oUz = o.take<char>((size_t)((mu + 3) / 4 * 4) * n * Tsz), oUuc = o.take<int>((size_t)mu * kMaxU);
+  const int ld = pad4(n);
+  const size_t oUz = o.take<char>((size_t)mu * ld * Tsz), oUuc = o.take<int>((size_t)mu * kMaxU);
   const size_t oUuv = o.take<char>((size_t)mu * kMaxU * Tsz), oUul = o.take<int>(mu);
   const size_t oG = o.take<double>((size_t)kMaxUpd * kMaxUpd);
-  const size_t oV = o.take<char>((size_t)(m + 1) * n * Tsz), oZk = o.take<char>((size_t)m * n * Tsz);
+  const size_t oV = o.take<char>((size_t)(m + 1) * ld * Tsz), oZk = o.take<char>((size_t)m * ld * Tsz);
   const size_t oTv = o.take<char>((size_t)3 * n * Tsz), oX = o.take<double>(n), oRr = o.take<double>(n);
   const size_t oPac = o.take<int>(cap), oPav = o.take<double>(cap), oPuc = o.take<int>(kMaxU);
   const size_t oPuv = o.take<double>(kMaxU), oMeta = o.take<int4>(n + 1), oLnc = o.take<int>(n + 1);
@@ -164,7 +165,20 @@ extern "C" vmc_status vmc_ratio_noalloc(const vmc_system* sys, const vmc_solver_
   const size_t oUh = o.take<double2>(n);
   const size_t oExl = o.take<int>(n), oExc = o.take<int>((size_t)n * exmax), oExv = o.take<double>((size_t)n * exmax);
   const size_t oCtl = o.take<Ctl>(1), oW = o.take<Walker>(1);
-  const size_t used = o.off;
+  size_t used = o.off;
+  // the transposed copy of the slots only where it fits: no system is refused for it
+  size_t oEc = 0, oEv = 0, oEf = 0;
+  bool ell = false;
+  if (n < 0x10000) {
+    Off t = o;
+    oEc = t.take<unsigned short>((size_t)cap * ld);
+    oEv = t.take<double>((size_t)cap * ld);
+    oEf = t.take<float>(fp64 ? 0 : (size_t)cap * ld);
+    if (t.off <= kNoAllocBytes) {
+      ell = true;
+      used = t.off;
+    }
+  }
   if (used > kNoAllocBytes)
     return fail(VMC_ERR_CAPACITY, "system too large for the no-allocation scratch: needs " + std::to_string(used) +
                                       " bytes, the fixed maximum is " + std::to_string(kNoAllocBytes));
@@ -176,12 +190,17 @@ extern "C" vmc_status vmc_ratio_noalloc(const vmc_system* sys, const vmc_solver_
 
   Walker W;
   std::memset(&W, 0, sizeof(W));
-  W.n = n; W.K = sys->K; W.lattice = sys->lattice; W.cap = cap; W.capLU = capLU; W.m = m; W.mu = mu; W.mu4 = (mu + 3) / 4 * 4; W.per = lay.per;
+  W.n = n; W.K = sys->K; W.lattice = sys->lattice; W.cap = cap; W.capLU = capLU; W.m = m; W.mu = mu; W.ld = ld; W.per = lay.per;
   W.a = sys->a; W.kappa = sys->kappa; W.rc = sys->r_c; W.rc2 = sys->r_c * sys->r_c; W.L = sys->K * sys->a;
   W.Z = (const double*)(base + oZ); W.col_of_orb = (const int*)(base + oCO); W.orb_of_col = (const int*)(base + oOC);
   W.R = (double*)(base + oR); W.row_of_part = (int*)(base + oRP); W.part_of_row = (int*)(base + oPR);
   W.a_col = (int*)(base + oAc); W.a_val = (double*)(base + oAv); W.a_val32 = (float*)(base + oAv32);
   W.a_len = (int*)(base + oAl);
+  if (ell) {
+    W.ell_col = (unsigned short*)(base + oEc);
+    W.ell_val = (double*)(base + oEv);
+    if (!fp64) W.ell_val32 = (float*)(base + oEf);
+  }
   W.l_col = (int*)(base + oLc); W.l_val64 = (double*)(base + oLv); W.lstream = base + oLs; W.l_len = (int*)(base + oLl);
   W.u_col = (int*)(base + oUc); W.u_val64 = (double*)(base + oUv); W.sbytes = sbytes; W.ustream = W.lstream + sbytes; W.u_len = (int*)(base + oUl);
   W.u_dinv64 = (double*)(base + oUd);
@@ -229,7 +248,7 @@ extern "C" vmc_status vmc_ratio_noalloc(const vmc_system* sys, const vmc_solver_
   const int budget = optin - stat;
   plan_smem(ybytes, budget, P, p.trisolve == 1);
   if (!P.y_smem && ybytes != ybytes1) plan_smem(ybytes1, budget, P, p.trisolve == 1);
-  const LaunchCfg L{s, p.block_threads ? p.block_threads : 256, fp64, (size_t)P.dsm_bytes};
+  const LaunchCfg L{s, p.block_threads ? p.block_threads : 256, fp64, (size_t)P.dsm_bytes, 1};
 
   // clear the part of the scratch this call uses, then fill the inputs
   e = cudaMemsetAsync(base, 0, used, s);

@@ -93,18 +93,22 @@ __device__ __noinline__ int ilutp_warp(const Walker& w, const Params& P, Shared&
     ucv = (T*)(ucc + ucap);
   }
   if (lbits) {
+#pragma unroll 1
     for (int i = lane; i < nwords; i += 32) lbits[i] = 0u;
+#pragma unroll 1
     for (int i = lane; i < nsum; i += 32) lsum[i] = 0u;
   }
   int p = P.lfil_extra;
   if (p < 0) {
     long long tot = 0;
+#pragma unroll 1
     for (int i = lane; i < n; i += 32) tot += w.a_len[i];
     tot = warp_sum_ll(tot);
     p = (int)((tot + 2LL * n - 1) / (2LL * n));  // ceil(avg nnz per row / 2)
   }
   p = min(p, (capLU - 2) / 2);
   const int pk = max(0, min(p, capLU - 2 - cap));  // never exceeds the row capacity
+#pragma unroll 1
   for (int i = lane; i < n; i += 32) {
     w.perm[i] = i; iperm[i] = i; wpos[i] = -1; wrow[i] = (T)0; levl[i] = 0;
   }
@@ -112,6 +116,7 @@ __device__ __noinline__ int ilutp_warp(const Walker& w, const Params& P, Shared&
   int npiv = 0, flags = 0;
   long long n_elim = 0, n_cand = 0;
   double nnz = 0.0;
+#pragma unroll 1
   for (int r = 0; r < n; ++r) {
     const int part = w.part_of_row[r];
     const int len = w.a_len[part];
@@ -119,6 +124,7 @@ __device__ __noinline__ int ilutp_warp(const Walker& w, const Params& P, Shared&
     const double* av = w.a_val + (size_t)part * cap;
     double ss = 0.0;
     int nl = 0, nu = 0;
+#pragma unroll 1
     for (int t = lane; t < len; t += 32) {
       const int f = iperm[ac[t]];
       const double v = av[t];
@@ -153,6 +159,7 @@ __device__ __noinline__ int ilutp_warp(const Walker& w, const Params& P, Shared&
           best = (w0 << 5) + __ffs(cur) - 1;
         } else {
           const int s0 = (w0 + 1) >> 5;  // summary word holding bitmap word w0 + 1
+#pragma unroll 1
           for (int sb = s0; sb < nsum && best == 0x7fffffff; sb += 32) {
             const int si = sb + lane;
             unsigned sv = si < nsum ? lsum[si] : 0u;
@@ -168,6 +175,7 @@ __device__ __noinline__ int ilutp_warp(const Walker& w, const Params& P, Shared&
         }
         if (best >= r) best = 0x7fffffff;
       } else {
+#pragma unroll 1
         for (int t = lane; t < cnt; t += 32) {
           const int f = sh.nz[t];
           if (f > last && f < r && f < best) best = f;
@@ -187,6 +195,7 @@ __device__ __noinline__ int ilutp_warp(const Walker& w, const Params& P, Shared&
       if (lane == 0) wrow[best] = wk;
       const int ul = ulen_a[best];
       const int ub = uoff ? uoff[best] : -1;
+#pragma unroll 1
       for (int base = 0; base < ul; base += 32) {
         const int t = base + lane;
         const bool valid = t < ul;
@@ -222,6 +231,7 @@ __device__ __noinline__ int ilutp_warp(const Walker& w, const Params& P, Shared&
     // --- L part: keep the nl + p largest multipliers ---
     T* selv = reinterpret_cast<T*>(sh.selV);
     int cL = 0;
+#pragma unroll 1
     for (int base = 0; base < cnt; base += 32) {
       const int t = base + lane;
       bool c = false;
@@ -238,6 +248,7 @@ __device__ __noinline__ int ilutp_warp(const Walker& w, const Params& P, Shared&
     const int keepL = nl + pk;
     select_topk<T>(sh, cL, keepL);
     int nL = 0, levmax = -1;
+#pragma unroll 1
     for (int base = 0; base < cL; base += 32) {
       const int e = base + lane;
       const bool k = e < cL && sh.selK[e];
@@ -256,6 +267,7 @@ __device__ __noinline__ int ilutp_warp(const Walker& w, const Params& P, Shared&
     // --- U part: entries above threshold, keep the nu + p largest ---
     T dval = wpos[r] >= 0 ? wrow[r] : (T)0;
     int cU = 0;
+#pragma unroll 1
     for (int base = 0; base < cnt; base += 32) {
       const int t = base + lane;
       bool c = false;
@@ -350,6 +362,7 @@ __device__ __noinline__ int ilutp_warp(const Walker& w, const Params& P, Shared&
     }
     nnz += (double)(nL + nU + 1);
     // clear the working row (and the pending-label bitmaps)
+#pragma unroll 1
     for (int t = lane; t < cnt; t += 32) {
       const int f = sh.nz[t];
       wpos[f] = -1;
@@ -360,13 +373,16 @@ __device__ __noinline__ int ilutp_warp(const Walker& w, const Params& P, Shared&
   }
   __syncwarp();
   if (sm_work)
+#pragma unroll 1
     for (int i = lane; i < n; i += 32) w.iperm[i] = iperm[i];
   if (sm_rows) {
+#pragma unroll 1
     for (int i = lane; i < n; i += 32) { w.u_dinv64[i] = (double)udinv[i]; w.u_len[i] = ulen_a[i]; w.lev_l[i] = levl[i]; }
   } else if (sizeof(T) != sizeof(double)) {
     // udinv aliased the global FP64 array as T values: widen in place, back to front
     __syncwarp();
     if (lane == 0)
+#pragma unroll 1
       for (int i = n - 1; i >= 0; --i) w.u_dinv64[i] = (double)udinv[i];
   }
   __syncwarp();
@@ -401,6 +417,7 @@ __device__ __forceinline__ IluSm ilu_sm_plan(int n, size_t dbytes) {
   pl.ok = 0;
   if (n > 65535) return pl;
   const unsigned nwords = (n + 31) >> 5, nsum = (nwords + 31) >> 5;
+#pragma unroll 1
   for (int lg = 12; lg >= 11; --lg) {
     const unsigned HS = 1u << lg, maxc = min((int)(HS / 2), kMaxRowNZ);
     unsigned o = 0;
@@ -451,14 +468,19 @@ __device__ __noinline__ int ilutp_warp_hash(const Walker& w, const Params& P, Sh
   int ufill = 0;
   const int HS = pl.HS, hmask = HS - 1, hshift = 32 - pl.lgHS, MAXC = pl.maxc;
   const int nwords = (n + 31) >> 5, nsum = (nwords + 31) >> 5;
+#pragma unroll 1
   for (int i = lane; i < nwords; i += 32) lbits[i] = 0u;
+#pragma unroll 1
   for (int i = lane; i < nsum; i += 32) lsum[i] = 0u;
+#pragma unroll 1
   for (int i = lane; i < HS; i += 32) hkey[i] = -1;
+#pragma unroll 1
   for (int i = lane; i < n; i += 32) { w.perm[i] = i; ip[i] = (unsigned short)i; w.lev_l[i] = 0; }
   __syncwarp();
   int p = P.lfil_extra;
   if (p < 0) {
     long long tot = 0;
+#pragma unroll 1
     for (int i = lane; i < n; i += 32) tot += w.a_len[i];
     tot = warp_sum_ll(tot);
     p = (int)((tot + 2LL * n - 1) / (2LL * n));  // ceil(avg nnz per row / 2)
@@ -472,6 +494,7 @@ __device__ __noinline__ int ilutp_warp_hash(const Walker& w, const Params& P, Sh
   // index of label f in the working row, or -1 (every lane the same)
   auto find = [&](int f) -> int {
     int h = hash_of(f);
+#pragma unroll 1
     for (int probe = 0; probe < HS; ++probe) {
       const int k = hkey[h];
       if (k == f) { const int t = hidx[h]; return t == 0xFFFF ? -1 : t; }
@@ -480,6 +503,7 @@ __device__ __noinline__ int ilutp_warp_hash(const Walker& w, const Params& P, Sh
     }
     return -1;
   };
+#pragma unroll 1
   for (int r = 0; r < n; ++r) {
     const int part = w.part_of_row[r];
     const int len = w.a_len[part];
@@ -487,10 +511,12 @@ __device__ __noinline__ int ilutp_warp_hash(const Walker& w, const Params& P, Sh
     const double* av = w.a_val + (size_t)part * cap;
     double ss = 0.0;
     int nl = 0, nu = 0;
+#pragma unroll 1
     for (int t = lane; t < len; t += 32) {  // distinct labels: plain inserts
       const int f = ip[ac[t]];
       const double v = av[t];
       int h = hash_of(f);
+#pragma unroll 1
       for (int probe = 0; probe < HS; ++probe) {
         if (atomicCAS(&hkey[h], -1, f) == -1) break;
         h = (h + 1) & hmask;
@@ -527,6 +553,7 @@ __device__ __noinline__ int ilutp_warp_hash(const Walker& w, const Params& P, Sh
           best = (w0 << 5) + __ffs(cur) - 1;
         } else {
           const int s0 = (w0 + 1) >> 5;  // summary word holding bitmap word w0 + 1
+#pragma unroll 1
           for (int sb = s0; sb < nsum && best == 0x7fffffff; sb += 32) {
             const int si = sb + lane;
             unsigned sv = si < nsum ? lsum[si] : 0u;
@@ -571,6 +598,7 @@ __device__ __noinline__ int ilutp_warp_hash(const Walker& w, const Params& P, Sh
         continue;
       }
       if (lane == 0) wv[tb] = wk;
+#pragma unroll 1
       for (int base = 0; base < ul; base += 32) {
         const int t = base + lane;
         const bool valid = t < ul;
@@ -585,6 +613,7 @@ __device__ __noinline__ int ilutp_warp_hash(const Walker& w, const Params& P, Sh
           else { c = w.u_col[(size_t)best * capLU + t]; v = (T)w.u_val64[(size_t)best * capLU + t]; }
           f = ip[c];
           h = hash_of(f);
+#pragma unroll 1
           for (int probe = 0; probe < HS; ++probe) {
             const int k = hkey[h];
             if (k == f) { ex = hidx[h]; break; }
@@ -623,6 +652,7 @@ __device__ __noinline__ int ilutp_warp_hash(const Walker& w, const Params& P, Sh
     // --- L part: keep the nl + p largest multipliers ---
     T* selv = reinterpret_cast<T*>(sh.selV);
     int cL = 0;
+#pragma unroll 1
     for (int base = 0; base < cnt; base += 32) {
       const int t = base + lane;
       bool c = false;
@@ -639,6 +669,7 @@ __device__ __noinline__ int ilutp_warp_hash(const Walker& w, const Params& P, Sh
     const int keepL = nl + pk;
     select_topk<T>(sh, cL, keepL);
     int nL = 0, levmax = -1;
+#pragma unroll 1
     for (int base = 0; base < cL; base += 32) {
       const int e = base + lane;
       const bool k = e < cL && sh.selK[e];
@@ -658,6 +689,7 @@ __device__ __noinline__ int ilutp_warp_hash(const Walker& w, const Params& P, Sh
     const int td = find(r);
     T dval = td >= 0 ? wv[td] : (T)0;
     int cU = 0;
+#pragma unroll 1
     for (int base = 0; base < cnt; base += 32) {
       const int t = base + lane;
       bool c = false;
@@ -756,15 +788,18 @@ __device__ __noinline__ int ilutp_warp_hash(const Walker& w, const Params& P, Sh
     if (cache && ufill + nU <= ucap) ufill += nU;
     nnz += (double)(nL + nU + 1);
     // clear the working row (and the pending-label bitmaps)
+#pragma unroll 1
     for (int t = lane; t < cnt; t += 32) {
       const int f = sh.nz[t];
       hkey[hslot[t]] = -1;
       if (f < r) { lbits[f >> 5] = 0u; lsum[f >> 10] = 0u; }
     }
     if (flags & 2)  // keys past the capacity have no slot record: clear the whole table
+#pragma unroll 1
       for (int i = lane; i < HS; i += 32) hkey[i] = -1;
     __syncwarp();
   }
+#pragma unroll 1
   for (int i = lane; i < n; i += 32) w.iperm[i] = ip[i];
   __syncwarp();
   if (lane == 0) { w.ctl->ilu_rows += n; w.ctl->ilu_elims += n_elim; w.ctl->ilu_cand += n_cand; }
@@ -804,8 +839,10 @@ __device__ int build_stream(const Walker& w, const Params& P, bool upper, int nl
   // dependent chain short; FP64 takes more (8), because every lane-group reduction step
   // is an FP64 add and GB300's FP64 pipe issues few per clock.  Packed as
   // entries | gs << 28 (entries < 2^28 for K <= 64).
+#pragma unroll 1
   for (int lev = wid; lev < nlev; lev += nw) {
     int e = 0, ml = 0;
+#pragma unroll 1
     for (int q = lptr[lev] + lane; q < lptr[lev + 1]; q += 32) {
       const int L = len[rows[q]];
       e += L;
@@ -823,6 +860,7 @@ __device__ int build_stream(const Walker& w, const Params& P, bool upper, int nl
     int nch = 0, nseg = 0;
     int cs = 0, cr = 0, ce = 0;  // open chunk: segments, rows, entries
     int c_seg0 = 0;
+#pragma unroll 1
     for (int lev = 0; lev < nlev; ++lev) {
       int q = lptr[lev];
       const int qe = lptr[lev + 1];
@@ -872,12 +910,15 @@ __device__ int build_stream(const Walker& w, const Params& P, bool upper, int nl
   }
   __syncthreads();
   const int nch_total = sh.iflag[2];
+#pragma unroll 1
   for (int c = tid; c < nch_total; c += nt) tab[c].y = w.lvl_cur[c];
   __syncthreads();
   block_scan_inplace(w.lvl_cur, nch_total, sh);
+#pragma unroll 1
   for (int c = tid; c < nch_total; c += nt) tab[c].x = w.lvl_cur[c];
   __syncthreads();
   // fill the chunks, one warp per chunk
+#pragma unroll 1
   for (int c = wid; c < nch_total; c += nw) {
     const int4 cm = w.chunk_meta[c];
     const int seg0 = cm.x, nseg = cm.y, nr = cm.z, ne = cm.w;
@@ -891,10 +932,12 @@ __device__ int build_stream(const Walker& w, const Params& P, bool upper, int nl
     if (lane == 0) *(int4*)base = make_int4(nseg, nr, ne, 0);
     if (lane < kMaxSlots) ((int2*)(base + 16))[lane] = c + 1 + lane < nch_total ? tab[c + 1 + lane] : make_int2(0, 0);
     int rbase = 0, carry = 0;
+#pragma unroll 1
     for (int sgi = 0; sgi < nseg; ++sgi) {
       const int4 sm = w.seg_meta[seg0 + sgi];
       const int q0 = sm.x, sr = sm.y;
       if (lane == 0) seg[sgi] = make_int4(rbase, sr, sm.w & 0xff, sm.w >> 8);
+#pragma unroll 1
       for (int b0 = 0; b0 < sr; b0 += 32) {
         const int i = b0 + lane;
         const int r = i < sr ? rows[q0 + i] : 0;
@@ -916,9 +959,11 @@ __device__ int build_stream(const Walker& w, const Params& P, bool upper, int nl
     }
     if (lane == 0) st[nr] = carry;
     __syncwarp();
+#pragma unroll 1
     for (int i = 0; i < nr; ++i) {
       const int r = rws[i];
       const int b = st[i], L = st[i + 1] - b;
+#pragma unroll 1
       for (int t = lane; t < L; t += 32) {
         cl[b + t] = colv[(size_t)r * capLU + t];
         vl[b + t] = (T)valv[(size_t)r * capLU + t];
@@ -945,6 +990,7 @@ static __device__ __noinline__ void row_levels(const int* len, const int* col, i
   };
 #pragma unroll
   for (int k = 0; k < kAhead; ++k) load(k, k);
+#pragma unroll 1
   for (int i0 = 0; i0 < n; i0 += kAhead) {
 #pragma unroll
     for (int k = 0; k < kAhead; ++k) {
@@ -953,6 +999,7 @@ static __device__ __noinline__ void row_levels(const int* len, const int* col, i
       int lv = -1;
       if (lane < L[k]) lv = lev[c0[k]];
       if (lane + 32 < L[k]) lv = max(lv, lev[c1[k]]);
+#pragma unroll 1
       for (int t = lane + 64; t < L[k]; t += 32) lv = max(lv, lev[col[(size_t)row(i) * capLU + t]]);
       lv = __reduce_max_sync(0xffffffffu, lv);
       if (lane == 0) lev[row(i)] = lv + 1;
@@ -966,24 +1013,32 @@ static __device__ __noinline__ void row_levels(const int* len, const int* col, i
 static __device__ __noinline__ void level_sets(const Walker& w, int nll, int nlu) {
   const int n = w.n, tid = threadIdx.x, nt = blockDim.x;
   __syncthreads();
+#pragma unroll 1
   for (int q = tid; q <= n; q += nt) { w.l_lvl_ptr[q] = 0; w.u_lvl_ptr[q] = 0; }
   __syncthreads();
+#pragma unroll 1
   for (int r = tid; r < n; r += nt) {
     atomicAdd(&w.l_lvl_ptr[w.lev_l[r] + 1], 1);
     atomicAdd(&w.u_lvl_ptr[w.lev_u[r] + 1], 1);
   }
   __syncthreads();
   if (tid == 0) {
+#pragma unroll 1
     for (int q = 0; q < nll; ++q) w.l_lvl_ptr[q + 1] += w.l_lvl_ptr[q];
+#pragma unroll 1
     for (int q = 0; q < nlu; ++q) w.u_lvl_ptr[q + 1] += w.u_lvl_ptr[q];
   }
   __syncthreads();
+#pragma unroll 1
   for (int q = tid; q < nll; q += nt) w.lvl_cur[q] = w.l_lvl_ptr[q];
   __syncthreads();
+#pragma unroll 1
   for (int r = tid; r < n; r += nt) w.l_lvl_rows[atomicAdd(&w.lvl_cur[w.lev_l[r]], 1)] = r;
   __syncthreads();
+#pragma unroll 1
   for (int q = tid; q < nlu; q += nt) w.lvl_cur[q] = w.u_lvl_ptr[q];
   __syncthreads();
+#pragma unroll 1
   for (int r = tid; r < n; r += nt) w.u_lvl_rows[atomicAdd(&w.lvl_cur[w.lev_u[r]], 1)] = r;
   __syncthreads();
 }
@@ -1011,6 +1066,7 @@ __device__ __noinline__ void level_streams(const Walker& w, const Params& P, int
 template <typename T>
 __device__ __noinline__ void relabel_and_levels(const Walker& w, const Params& P, Shared& sh) {
   const int n = w.n, tid = threadIdx.x, nt = blockDim.x, capLU = w.capLU;
+#pragma unroll 1
   for (int idx = tid; idx < n * capLU; idx += nt) {
     const int r = idx / capLU, t = idx - r * capLU;
     if (t < w.u_len[r]) w.u_col[idx] = w.iperm[w.u_col[idx]];
@@ -1023,12 +1079,14 @@ __device__ __noinline__ void relabel_and_levels(const Walker& w, const Params& P
     int* lev = sm ? (int*)dyn_smem() + (up ? 0 : n) : glob;
     row_levels(up ? w.u_len : w.l_len, up ? w.u_col : w.l_col, n, capLU, up, lev);
     if (sm)
+#pragma unroll 1
       for (int r = tid & 31; r < n; r += 32) glob[r] = lev[r];
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // scratch is reused by bulk copies
   }
   __syncthreads();
   // level counts
   int mlv = 0, muv = 0;
+#pragma unroll 1
   for (int r = tid; r < n; r += nt) { mlv = max(mlv, w.lev_l[r]); muv = max(muv, w.lev_u[r]); }
   const int nll = block_max_int(mlv, sh) + 1;
   const int nlu = block_max_int(muv, sh) + 1;
@@ -1106,6 +1164,7 @@ __device__ __noinline__ int factor_block(const Walker& w, const Params& P, Share
   if (threadIdx.x == 0) w.ctl->cyc[PH_LEVELS] += clock64() - tl;
   if (threadIdx.x < 32) {
     long long tot = 0;
+#pragma unroll 1
     for (int i = threadIdx.x; i < w.n; i += 32) tot += w.a_len[i];
     tot = warp_sum_ll(tot);
     if (threadIdx.x == 0) {

@@ -33,22 +33,32 @@ struct Nearest {
 // margin(d): twice the error of FP32 distances^2 around d.  Returns the position, or -1.
 template <typename Each, typename Exact, typename Margin>
 __device__ __forceinline__ int nearest_warp(float limit, Each each, Exact exact, Margin margin) {
-  float m = 3e38f;
-  each([&](int, float d, int) { m = fminf(m, d); });
-  m = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(m)));  // d >= 0
-  const float thr = m + margin(m);
-  if (!(thr < limit)) return -1;
+  float m = 3e38f, thr = 0.0f;
   int cnt = 0, pos = 0x7fffffff;
-  each([&](int p, float d, int) {
-    if (d <= thr) { ++cnt; pos = p; }
-  });
-  if (__reduce_add_sync(0xffffffffu, cnt) == 1) return __reduce_min_sync(0xffffffffu, pos);
   Nearest b{1e300, 0x7fffffff};
-  each([&](int p, float d, int id) {
-    if (d > thr) return;
-    const double x = exact(id);
-    if (x < b.d || (x == b.d && p < b.pos)) { b.d = x; b.pos = p; }
-  });
+#pragma unroll 1
+  for (int pass = 0; pass < 3; ++pass) {  // the least FP32 distance; who is near it; FP64 among those
+    each([&](int p, float d, int id) {
+      if (pass == 0) {
+        m = fminf(m, d);
+      } else if (d <= thr) {
+        if (pass == 1) {
+          ++cnt;
+          pos = p;
+        } else {
+          const double x = exact(id);
+          if (x < b.d || (x == b.d && p < b.pos)) { b.d = x; b.pos = p; }
+        }
+      }
+    });
+    if (pass == 0) {
+      m = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(m)));  // d >= 0
+      thr = m + margin(m);
+      if (!(thr < limit)) return -1;
+    } else if (pass == 1) {
+      if (__reduce_add_sync(0xffffffffu, cnt) == 1) return __reduce_min_sync(0xffffffffu, pos);
+    }
+  }
 #pragma unroll
   for (int o = 16; o; o >>= 1) {
     const double d2 = __shfl_xor_sync(0xffffffffu, b.d, o);
@@ -68,6 +78,7 @@ __device__ __noinline__ void reorder_search(const Walker& w, I* pos_orb, I* pos_
   // the factor 0.9999 on the search limits covers (K <= 64)
   const float inva = 1.0f / (float)w.a;
   auto cell_axis = [&](float x) { return min(K - 1, max(0, (int)floorf(x * inva))); };
+#pragma unroll 1
   for (int c = tid; c < n; c += nt) {
     const int p = w.part_of_row[c], o = w.orb_of_col[c];
     part_at[c] = (I)p;
@@ -75,8 +86,10 @@ __device__ __noinline__ void reorder_search(const Walker& w, I* pos_orb, I* pos_
     pos_part[p] = (I)c;
     pos_orb[o] = (I)c;
   }
+#pragma unroll 1
   for (int c = tid; c < K * K * K; c += nt) head[c] = kNone;
   __syncthreads();
+#pragma unroll 1
   for (int p = tid; p < n; p += nt) {
     const double* r = w.R + 3 * p;
     const int c = cell_axis((float)r[0]) + K * (cell_axis((float)r[1]) + K * cell_axis((float)r[2]));
@@ -107,6 +120,7 @@ __device__ __noinline__ void reorder_search(const Walker& w, I* pos_orb, I* pos_
       z = a * ((float)(c / K) + off);
     };
     auto wrap_cell = [&](int c) { return c < 0 ? c + K : (c >= K ? c - K : c); };
+#pragma unroll 1
     for (int i = 0; i < n - 1; ++i) {
       const int p = part_at[i];
       const double rp[3] = {w.R[3 * p], w.R[3 * p + 1], w.R[3 * p + 2]};
@@ -115,9 +129,11 @@ __device__ __noinline__ void reorder_search(const Walker& w, I* pos_orb, I* pos_
       int bj = -1;
       if (!few) {
         const int cx = cell_axis(px), cy = cell_axis(py), cz = cell_axis(pz);
+#pragma unroll 1
         for (int rad = 1; rad <= 3 && 2 * rad + 1 <= K && bj < 0; ++rad) {
           const int s = 2 * rad + 1, tot = s * s * s * per;
           auto each = [&](auto f) {
+#pragma unroll 1
             for (int q = lane; q < tot; q += 32) {
               const int b = per == 2 ? (q & 1) : 0;
               int t = per == 2 ? q >> 1 : q;
@@ -138,6 +154,7 @@ __device__ __noinline__ void reorder_search(const Walker& w, I* pos_orb, I* pos_
       }
       if (bj < 0) {
         auto each = [&](auto f) {
+#pragma unroll 1
           for (int j = i + lane; j < n; j += 32) {
             const int o = orb_at[j];
             float x, y, z;
@@ -172,14 +189,17 @@ __device__ __noinline__ void reorder_search(const Walker& w, I* pos_orb, I* pos_
         const int cx = c % K;
         c /= K;
         const int cy = c % K, cz = c / K;
+#pragma unroll 1
         for (int rad = 1; rad <= 3 && 2 * rad + 1 <= K && bk < 0; ++rad) {
           const int s = 2 * rad + 1, tot = s * s * s;
           auto each = [&](auto f) {
+#pragma unroll 1
             for (int q = lane; q < tot; q += 32) {
               int t = q;
               const int x = wrap_cell(cx - rad + t % s);
               t /= s;
               const int y = wrap_cell(cy - rad + t % s), z = wrap_cell(cz - rad + t / s);
+#pragma unroll 1
               for (int k = head[x + K * (y + K * z)]; k != kNone; k = (int)next[k]) {
                 const int g = (int)pos_part[k];
                 if (g >= i) f(g, part_dist(k), k);
@@ -193,6 +213,7 @@ __device__ __noinline__ void reorder_search(const Walker& w, I* pos_orb, I* pos_
       }
       if (bk < 0) {
         auto each = [&](auto f) {
+#pragma unroll 1
           for (int k = i + lane; k < n; k += 32) {
             const int q = part_at[k];
             f(k, part_dist(q), q);
@@ -210,6 +231,7 @@ __device__ __noinline__ void reorder_search(const Walker& w, I* pos_orb, I* pos_
     }
   }
   __syncthreads();
+#pragma unroll 1
   for (int g = tid; g < n; g += nt) {
     const int c = w.col_of_orb[orb_at[g]];
     const int p = part_at[g];

@@ -24,16 +24,20 @@ __device__ __forceinline__ void select_topk(int* hist, B* bnd, unsigned char* se
                                             Label label) {
   const int lane = threadIdx.x & 31;
   if (c <= keep) {
+#pragma unroll 1
     for (int e = lane; e < c; e += 32) selK[e] = 1;
     __syncwarp();
     return;
   }
   int emax = 0;
+#pragma unroll 1
   for (int e = lane; e < c; e += 32) emax = max(emax, key_exp(key(e)));
   emax = __reduce_max_sync(0xffffffffu, emax);
   auto bin = [&](K k) { return min(63, emax - key_exp(k)); };
+#pragma unroll 1
   for (int b = lane; b < 64; b += 32) hist[b] = 0;
   __syncwarp();
+#pragma unroll 1
   for (int e = lane; e < c; e += 32) atomicAdd(&hist[bin(key(e))], 1);
   __syncwarp();
   // boundary bin bb: count(bins < bb) < keep <= count(bins <= bb)
@@ -54,6 +58,7 @@ __device__ __forceinline__ void select_topk(int* hist, B* bnd, unsigned char* se
   const int need = keep - below;  // entries to keep from the boundary bin
   // compact the boundary octave, decide the others
   int cb = 0;
+#pragma unroll 1
   for (int base = 0; base < c; base += 32) {
     const int e = base + lane;
     int b = 64;
@@ -68,11 +73,13 @@ __device__ __forceinline__ void select_topk(int* hist, B* bnd, unsigned char* se
   }
   __syncwarp();
   if (cb <= 256) {
+#pragma unroll 1
     for (int q = lane; q < cb; q += 32) {
       const int e = bnd[q];
       const K me = key(e);
       const int fe = label(e);
       int rank = 0;
+#pragma unroll 1
       for (int o = 0; o < cb; ++o) {
         const int eo = bnd[o];
         const K mo = key(eo);
@@ -81,11 +88,13 @@ __device__ __forceinline__ void select_topk(int* hist, B* bnd, unsigned char* se
       selK[e] = rank < need ? 1 : 0;
     }
   } else {
+#pragma unroll 1
     for (int e = lane; e < c; e += 32) {
       const K me = key(e);
       if (bin(me) != bb) continue;
       const int fe = label(e);
       int rank = 0;
+#pragma unroll 1
       for (int o = 0; o < c; ++o) {
         const K mo = key(o);
         if (bin(mo) != bb) continue;
