@@ -820,7 +820,7 @@ static vmc_status check_walker_status(vmc_ctx* ctx) {
 }
 
 static vmc_status setup_all(vmc_ctx* ctx, int w0, int nwalk) {
-  if (ctx->dense) CK(launch_dense_setup(cfg(ctx), ctx->dW + w0, nwalk), "dense setup kernel");
+  if (ctx->dense) CK(launch_dense_setup(cfg(ctx), ctx->dW + w0, nwalk, ctx->max_n), "dense setup kernel");
   else {
     Params P;
     const LaunchCfg L = factor_cfg(ctx, P);
@@ -1017,7 +1017,7 @@ static vmc_status enqueue_sweeps(vmc_ctx* ctx, int n_sweeps, double sigma, const
   const long long s0 = ctx->sweeps;
   const int eng = ctx->prm.engine;
   if (eng == VMC_ENGINE_DENSE_SM) {
-    CK(launch_dense_sweep(L, ctx->dW, ctx->nw, n_sweeps, s0, sigma, d_seeds, acc, ratio, ctx->prm.sm_refresh),
+    CK(launch_dense_sweep(L, ctx->dW, ctx->nw, ctx->max_n, n_sweeps, s0, sigma, d_seeds, acc, ratio, ctx->prm.sm_refresh),
        "dense sweep kernel");
   } else if (eng == VMC_ENGINE_PERSISTENT && ctx->pair) {
     if (++ctx->launch_seq <= 0) ctx->launch_seq = 1;

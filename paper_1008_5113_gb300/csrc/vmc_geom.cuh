@@ -72,7 +72,14 @@ __device__ __forceinline__ double wrap_box(double x, double L) {
   if (y >= L) y = __dsub_rn(y, L);
   return y;
 }
+// The plainly rounded d - L rint(d / L).  For |d| < L the quotient rounds to at most 1 in
+// magnitude and rint of it is 0 up to |d| = L / 2 (the quotient 1/2 itself rounds to even, and
+// the first |d| above L / 2 gives a quotient above 1/2), +-1 beyond: two integer compares of
+// the bit patterns in place of an FP64 division (440 cycles a warp; three a distance).
 __device__ __forceinline__ double min_image(double d, double L) {
+  const unsigned long long a = (unsigned long long)__double_as_longlong(d) & 0x7fffffffffffffffull;
+  if (a < (unsigned long long)__double_as_longlong(L))
+    return a > (unsigned long long)__double_as_longlong(0.5 * L) ? __dsub_rn(d, copysign(L, d)) : d;
   return __dsub_rn(d, __dmul_rn(L, rint(__ddiv_rn(d, L))));
 }
 __device__ __forceinline__ double dist2(const double* r, const double* z, double L) {
