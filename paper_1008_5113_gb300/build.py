@@ -1,6 +1,6 @@
 """In-tree build of the CUDA library ``libvmc.so`` for sm_103a (nvcc, no cmake).
 
-The translation units (the engine's kernels in FP64 and in FP32, in six parts each, the precision-independent
+The translation units (the engine's kernels in FP64 and in FP32, in seven parts each, the precision-independent
 launch entry points; C ABI + host layout; the allocation-free entry point; the dense
 reference engine) compile in parallel and are linked into
 ``paper_1008_5113_gb300/libvmc.so`` next to this file.
@@ -18,7 +18,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libvmc.so")
 GENCODE = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # (source, defines): the engine's kernels are compiled in parts, the longest first
-PARTS = [2, 1, 3, 4, 0, 5]
+PARTS = [1, 3, 4, 2, 6, 0, 5]
 SOURCES = [(f"vmc_engine_{p}.cu", [f"-DVMC_PART={k}"]) for k in PARTS for p in ("f32", "f64")]
 SOURCES += [(s, []) for s in ("vmc_engine.cu", "vmc_capi.cu", "vmc_noalloc.cu", "vmc_dense.cu")]
 

@@ -15,7 +15,7 @@
 //     column permutation perm/iperm, level sets and the chunk streams the triangular
 //     solves read (two such factor sets when a second CTA refactors in the background);
 //   * the chain of rank-one preconditioner updates (z_hat_s, u_s) of Sec. 3.2 Eq. 18
-//     with the small matrix G[s][t] = u_s^T z_hat_t;
+//     and the inverse of I + G, G[s][t] = u_s^T z_hat_t (u and the inverse with s fastest);
 //   * the Krylov basis V and preconditioned vectors Zk of GMRES (Sec. 3.2 Eq. 15).
 #pragma once
 #include <cstdint>

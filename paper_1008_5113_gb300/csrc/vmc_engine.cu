@@ -54,10 +54,16 @@ cudaError_t launch_sweep(const LaunchCfg& L, const Walker* W, int walker0, int n
 cudaError_t launch_sweep_pair(const LaunchCfg& L, const Walker* W, int walker0, int nwalk, const Params& P,
                               int n_sweeps, long long sweep0, double sigma, const uint64_t* seeds, uint8_t* acc,
                               double* ratio, int launch_id) {
-  return L.fp64 ? launch_sweep_pair_T<double>(L, W, walker0, nwalk, P, n_sweeps, sweep0, sigma, seeds, acc, ratio,
-                                              launch_id)
-                : launch_sweep_pair_T<float>(L, W, walker0, nwalk, P, n_sweeps, sweep0, sigma, seeds, acc, ratio,
-                                             launch_id);
+  // more pairs than SMs: two CTAs an SM, as the shared-memory plan has them
+  if (L.per_sm > 1)
+    return L.fp64 ? launch_sweep_pair_T<double, 2>(L, W, walker0, nwalk, P, n_sweeps, sweep0, sigma, seeds, acc, ratio,
+                                                   launch_id)
+                  : launch_sweep_pair_T<float, 2>(L, W, walker0, nwalk, P, n_sweeps, sweep0, sigma, seeds, acc, ratio,
+                                                  launch_id);
+  return L.fp64 ? launch_sweep_pair_T<double, 1>(L, W, walker0, nwalk, P, n_sweeps, sweep0, sigma, seeds, acc, ratio,
+                                                 launch_id)
+                : launch_sweep_pair_T<float, 1>(L, W, walker0, nwalk, P, n_sweeps, sweep0, sigma, seeds, acc, ratio,
+                                                launch_id);
 }
 // Advance / set the device-side sweep index of the replayed sweep graphs.
 __global__ void k_next_sweep(long long* sweep_dev) { *sweep_dev += 1; }

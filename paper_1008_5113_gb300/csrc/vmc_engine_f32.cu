@@ -13,7 +13,10 @@ template cudaError_t launch_accept_T<float>(const LaunchCfg&, const Walker*, int
 template cudaError_t launch_sweep_T<float>(const LaunchCfg&, const Walker*, int, int, const Params&, int, long long,
                                          double, const uint64_t*, uint8_t*, double*);
 #elif VMC_PART == 2
-template cudaError_t launch_sweep_pair_T<float>(const LaunchCfg&, const Walker*, int, int, const Params&, int,
+template cudaError_t launch_sweep_pair_T<float, 1>(const LaunchCfg&, const Walker*, int, int, const Params&, int,
+                                              long long, double, const uint64_t*, uint8_t*, double*, int);
+#elif VMC_PART == 6
+template cudaError_t launch_sweep_pair_T<float, 2>(const LaunchCfg&, const Walker*, int, int, const Params&, int,
                                               long long, double, const uint64_t*, uint8_t*, double*, int);
 #elif VMC_PART == 3
 template cudaError_t prepare_step_kernels_T<float>(const LaunchCfg&);

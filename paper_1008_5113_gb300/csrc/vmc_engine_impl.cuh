@@ -520,8 +520,8 @@ __global__ void __launch_bounds__(kMaxThreads, kPerSm) k_sweep(const Walker* __r
 // Persistent sweeps with background refactorisation: a cluster of two CTAs per walker,
 // rank 0 steps (as k_sweep), rank 1 factors (af_factor_loop).  launch_id: unique per
 // launch of this context, > 0.
-template <typename T>
-__global__ void __launch_bounds__(kMaxThreads, 1) k_sweep_pair(const Walker* __restrict__ W, int walker0, Params P_,
+template <typename T, int kPerSm>
+__global__ void __launch_bounds__(kMaxThreads, kPerSm) k_sweep_pair(const Walker* __restrict__ W, int walker0, Params P_,
                                                      int n_sweeps, long long sweep0, double sigma,
                                                      const uint64_t* __restrict__ seeds, uint8_t* acc_log,
                                                      double* ratio_log, int launch_id) {
@@ -847,7 +847,7 @@ cudaError_t launch_sweep_T(const LaunchCfg& L, const Walker* W, int walker0, int
                            long long sweep0, double sigma, const uint64_t* seeds, uint8_t* acc, double* ratio) {
   VMC_LAUNCH_PER_SM(k_sweep, nwalk, W, walker0, P, n_sweeps, sweep0, sigma, seeds, acc, ratio);
 }
-template <typename T>
+template <typename T, int kPerSm>
 cudaError_t launch_sweep_pair_T(const LaunchCfg& L, const Walker* W, int walker0, int nwalk, const Params& P,
                                 int n_sweeps, long long sweep0, double sigma, const uint64_t* seeds, uint8_t* acc,
                                 double* ratio, int launch_id) {
@@ -863,9 +863,9 @@ cudaError_t launch_sweep_pair_T(const LaunchCfg& L, const Walker* W, int walker0
   at[0].val.clusterDim.z = 1;
   lc.attrs = at;
   lc.numAttrs = 1;
-  cudaError_t e = prep(k_sweep_pair<T>, L);
+  cudaError_t e = prep(k_sweep_pair<T, kPerSm>, L);
   if (e != cudaSuccess) return e;
-  return cudaLaunchKernelEx(&lc, k_sweep_pair<T>, W, walker0, P, n_sweeps, sweep0, sigma, seeds, acc, ratio, launch_id);
+  return cudaLaunchKernelEx(&lc, k_sweep_pair<T, kPerSm>, W, walker0, P, n_sweeps, sweep0, sigma, seeds, acc, ratio, launch_id);
 }
 template <typename T>
 cudaError_t prepare_step_kernels_T(const LaunchCfg& L) { return L.per_sm > 1 ? prep(k_step<T, 2>, L) : prep(k_step<T, 1>, L); }

@@ -58,7 +58,7 @@ template <typename T> int kernel_static_smem_T();
 template <typename T>
 cudaError_t launch_sweep_T(const LaunchCfg& L, const Walker* W, int walker0, int nwalk, const Params& P, int n_sweeps,
                            long long sweep0, double sigma, const uint64_t* seeds, uint8_t* acc, double* ratio);
-template <typename T>
+template <typename T, int kPerSm>
 cudaError_t launch_sweep_pair_T(const LaunchCfg& L, const Walker* W, int walker0, int nwalk, const Params& P,
                                 int n_sweeps, long long sweep0, double sigma, const uint64_t* seeds, uint8_t* acc,
                                 double* ratio, int launch_id);
@@ -87,7 +87,7 @@ cudaError_t launch_bench_T(const LaunchCfg& L, const Walker* W, int nwalk, const
 // least four fit, else 8 KB.  Fills tri_sf, y_half, y_smem, y_bytes, ring_slots,
 // slot_bytes, dsm_bytes.
 void plan_smem(int ybytes, int budget, Params& P, bool allow_sf);
-// Entries of an expanded row of the grouped triangular solves (a multiple of 4).
+// Entries a row of the scratch of the blocked triangular solves (a multiple of 4).
 int expanded_row_cap(int capLU, int row_cap);
 // Bytes of one factor's stream buffer; a factor set has two side by side.
 size_t stream_bytes(int n, int capLU, int exmax);

@@ -1,9 +1,9 @@
 // vmc_krylov.cuh -- the per-move solve A_p z = e_r and the determinant ratio.
 //
 //   * M v = prod_s (I - z_hat_s u_s^T) Q (L U)^{-1} v                (Sec. 3.2 Eq. 18)
-//     forward/backward substitution level by level (rows of a level in parallel),
-//     then the column permutation Q, then the update chain fused into one pass:
-//     c_s = u_s^T w_0 - sum_{t<s} G[s][t] c_t,  w = w_0 - sum_s z_hat_s c_s.
+//     the triangular solves from task streams (vmc_blocks.cuh) or, from chunk streams, level
+//     by level, then the column permutation Q, then the update chain:
+//     c = (I + G)^{-1} (u_s^T w_0)_s,  w = w_0 - sum_s z_hat_s c_s.
 //   * right-preconditioned GMRES(m) on A_p M (Sec. 3.2 Eq. 15) with classical
 //     Gram-Schmidt (reorthogonalised when it cancels), Givens rotations, and the effective stability
 //     N = max_j ||v_j - A_p M v_j||_2 over the Arnoldi vectors (Sec. 3.1 Eq. 10),
