@@ -74,3 +74,27 @@ def test_apply_matches_dense_solves(vmc, prec, K, lat, walkers, kw):
         assert st["groups_L"] <= 2 * -(-n // 16) and st["groups_U"] <= 2 * -(-n // 16)
     else:
         assert st["groups_L"] == st["levels_L"] and st["groups_U"] == st["levels_U"]
+
+
+def test_more_walker_pairs_than_sms(vmc):
+    """Background refactorisation asked for with more pairs than SMs (two CTAs an SM, two
+    tasks or more a warp in half an SM's shared memory): the first moves of two walkers against
+    the oracle's chains."""
+    K, walkers, moves = 5, 160, 40
+    seeds = list(range(1, walkers + 1))
+    ctx = vmc.vmc_create([(K, 0, 1.0, 2.0, 1.5)] * walkers,
+                         vmc.params(precision=1, refactor_lag=4, max_updates=8, sweep_moves=moves))
+    try:
+        vmc.vmc_init_positions(ctx, seeds, 0.1)
+        acc, rat = vmc.vmc_sweep(ctx, 1, 0.2, seeds)
+        st = vmc.vmc_get_stats(ctx, walkers - 1)
+    finally:
+        vmc.vmc_destroy(ctx)
+    assert st["async_lag"] == 4 and st["refactors_async"] > 0
+    s = O.system(K)
+    for w in (0, walkers - 1):
+        R0 = O.initial_positions(s, seeds[w], 0.1)
+        _, r_ref, a_ref, _ = O.chain(s, seeds[w], 0.2, R0, 1, max_steps=moves, solver=O.SOLVER_SHERMAN_MORRISON)
+        lo = w * K ** 3
+        assert np.array_equal(acc[lo:lo + moves], a_ref[:moves])
+        assert np.all(np.abs(rat[lo:lo + moves] - r_ref[:moves]) <= 1e-10 * np.maximum(np.abs(r_ref[:moves]), 1e-3))
