@@ -33,6 +33,16 @@ bool rows_fit_slot(int cap, int lfil_extra, int row_cap) {
   return chunk_bytes(1, 1, mx, 8, true) <= kSlotBytes && chunk_bytes_grouped(1, 1, mx, 8) <= kSlotBytes;
 }
 
+// Entries a row of a context's scratch for the inverses of the diagonal blocks.  It bounds the
+// rows of a block (block_rows), so without an explicit cap it has room for full ones, and the
+// streams are sized to match: a caller's cap stays the caller's.  n = 4096, fill limit that gave
+// blocks of 64 rows: 128 rows take the L and U solves of an iteration from 93 to 70 us, for
+// n x 64 more entries of scratch a factor set.
+static int block_scratch(int n, int capLU, int row_cap) {
+  const int c = expanded_row_cap(capLU, row_cap);
+  return row_cap > 0 ? c : std::max(c, n >= 2048 ? kMaxBlk : 64);
+}
+
 size_t stream_bytes(int n, int capLU, int exmax) {
   return ((size_t)n * (256 + 12 * (size_t)std::max(capLU, exmax)) + 255) & ~(size_t)255;
 }
@@ -460,7 +470,7 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     const int n = L.n, cap = L.cap, ld = pad4(n);
     const int pmax = p.lfil_extra >= 0 ? p.lfil_extra : (cap + 1) / 2;
     const int capLU = (cap + pmax + 2 + 3) / 4 * 4;  // rows of 16-byte multiples (bulk copies)
-    const int exmax = expanded_row_cap(capLU, p.trisolve_row_cap);
+    const int exb = block_scratch(n, capLU, p.trisolve_row_cap);
     auto& o = offs[w];
     o.push_back(cv.take<double>((size_t)n * 3));       // 0 Z
     o.push_back(cv.take<int>(n));                      // 1 col_of_orb
@@ -475,7 +485,7 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     o.push_back(cv.take<int>(n));                      // 9 a_len
     o.push_back(cv.take<int>((size_t)n * capLU));      // 10 l_col
     o.push_back(cv.take<double>((size_t)n * capLU));   // 11 l_val64
-    const size_t sbytes = stream_bytes(n, capLU, exmax);
+    const size_t sbytes = stream_bytes(n, capLU, exb);
     o.push_back(cv.take<unsigned char>(2 * sbytes));   // 12 lstream | ustream
     o.push_back(cv.take<int>(n));                      // 13 l_len
     o.push_back(cv.take<int>((size_t)n * capLU));      // 14 u_col
@@ -553,8 +563,8 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     if (ctx->pair) o.push_back(cv.take<double2>(n));
     for (int sset = 0; sset < (ctx->pair ? 2 : 1); ++sset) {  // inverses of the diagonal blocks of each factor set
       o.push_back(cv.take<int>(n));                      // ex_len
-      o.push_back(cv.take<int>((size_t)n * exmax));      // ex_col
-      o.push_back(cv.take<double>((size_t)n * exmax));   // ex_val
+      o.push_back(cv.take<int>((size_t)n * exb));        // ex_col
+      o.push_back(cv.take<double>((size_t)n * exb));     // ex_val
     }
     ell_off[w] = cv.take<unsigned short>(ell ? (size_t)cap * ld : 0);
     ell_off[n_walkers + w] = cv.take<double>(ell ? (size_t)cap * ld : 0);
@@ -641,7 +651,7 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     W.l_len = (int*)(A + o[13]);
     W.u_col = (int*)(A + o[14]);
     W.u_val64 = (double*)(A + o[15]);
-    W.sbytes = stream_bytes(W.n, W.capLU, expanded_row_cap(W.capLU, ctx->row_cap));
+    W.sbytes = stream_bytes(W.n, W.capLU, block_scratch(W.n, W.capLU, ctx->row_cap));
     W.ustream = W.lstream + W.sbytes;
     W.u_len = (int*)(A + o[17]);
     W.u_dinv64 = (double*)(A + o[18]);
@@ -680,7 +690,7 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     W.u_head = (double2*)(A + o[ctx->pair ? 82 : 50]);
     {
       const size_t e0 = ctx->pair ? 84 : 51;
-      W.exmax = expanded_row_cap(W.capLU, ctx->row_cap);
+      W.exmax = block_scratch(W.n, W.capLU, ctx->row_cap);
       W.ex_len = (int*)(A + o[e0]);
       W.ex_col = (int*)(A + o[e0 + 1]);
       W.ex_val = (double*)(A + o[e0 + 2]);

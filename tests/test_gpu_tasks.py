@@ -98,3 +98,32 @@ def test_more_walker_pairs_than_sms(vmc):
         lo = w * K ** 3
         assert np.array_equal(acc[lo:lo + moves], a_ref[:moves])
         assert np.all(np.abs(rat[lo:lo + moves] - r_ref[:moves]) <= 1e-10 * np.maximum(np.abs(r_ref[:moves]), 1e-3))
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("K,kw,B", [
+    (13, {}, 128),                                      # 2197 = 17 x 128 + 21
+    (13, dict(lfil_extra=0), 128),                      # shortest factor rows
+    (13, dict(lfil_extra=0, trisolve_row_cap=64), 64),  # a caller's cap bounds the blocks
+    (12, {}, 64),                                       # 1728: below the line
+])
+def test_rows_of_a_block(vmc, prec, K, kw, B):
+    """The blocks have their full rows whatever the fill limit, and the streams hold them
+    (the level-by-level fallback would take a step per level)."""
+    from scipy.linalg import solve_triangular
+    s = O.system(K, 0, 1.0, 2.0, 1.45)
+    n = K ** 3
+    ctx = vmc.vmc_create([(K, 0, 1.0, 2.0, 1.45)], vmc.params(precision=prec, **kw))
+    try:
+        vmc.vmc_set_positions(ctx, 0, O.initial_positions(s, 5, 0.2))
+        L, U, perm = vmc.vmc_get_factors(ctx, 0)
+        st = vmc.vmc_get_stats(ctx, 0)
+        v = np.random.default_rng(K).standard_normal(n)
+        z = vmc.vmc_apply_preconditioner(ctx, 0, v)
+    finally:
+        vmc.vmc_destroy(ctx)
+    ref = np.zeros(n)
+    ref[perm] = solve_triangular(U, solve_triangular(L, v, lower=True))  # substitution: the factors may be near singular
+    assert np.abs(z - ref).max() <= (1e-12 if prec == 0 else 1e-5) * np.abs(ref).max()
+    nb = -(-n // B)
+    assert nb <= st["groups_U"] <= 2 * nb and st["groups_L"] <= 2 * nb
