@@ -420,6 +420,11 @@ vmc_status vmc_kernel_bench(vmc_ctx* ctx, int which, int reps);
  * VMC_ERR_TIMEOUT when the wait gave up and reported it, as every bounded wait in the
  * engine does.  The context stays usable. */
 vmc_status vmc_check_wait_timeout(vmc_ctx* ctx);
+/* Failure detection check (tests): reorders and refactors walker w with a wait limit of 0
+ * between the rows that the ILUTP has in flight, so that a row's wait for the row before it
+ * runs out; returns VMC_ERR_TIMEOUT, the walker's status from then on until its positions
+ * are set again (VMC_OK where the factorisation has one row in flight and does not wait). */
+vmc_status vmc_check_factor_timeout(vmc_ctx* ctx, int walker);
 /* Philox4x32-10 on the device for n counters (host arrays ctr: 4n words, key: 2
  * words, out: 4n words): checks the device generator against its definition. */
 vmc_status vmc_philox_device(const uint32_t* ctr, const uint32_t* key, uint32_t* out, int n);

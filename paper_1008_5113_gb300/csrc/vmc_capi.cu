@@ -410,6 +410,7 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
   ctx->P.step_limit = p.sweep_moves;
   ctx->P.ilu_variant = p.ilutp_variant;
   ctx->P.warp_rows = p.trisolve_warp_rows;
+  ctx->P.ilu_wait_ns = kIluWaitNs;
   ctx->row_cap = p.trisolve_row_cap;
   ctx->P.lane_entries = p.trisolve_lane_entries > 0 ? p.trisolve_lane_entries : (ctx->fp64 ? 8 : 2);
   ctx->P.tri_group = p.trisolve == 1 ? 1 : std::max(1, p.trisolve_group);  // the sync-free solves read levels
@@ -1320,6 +1321,18 @@ extern "C" vmc_status vmc_check_wait_timeout(vmc_ctx* ctx) {
   if (e != cudaSuccess) return cuda_fail(ctx, e, "wait-timeout kernel");
   if (h != ST_TIMEOUT) return fail(ctx, VMC_ERR_STATE, "bounded wait did not report a timeout");
   return fail(ctx, VMC_ERR_TIMEOUT, "device wait gave up after its time limit (expected)");
+}
+
+extern "C" vmc_status vmc_check_factor_timeout(vmc_ctx* ctx, int walker) {
+  if (ctx && ctx->dense) return fail(ctx, VMC_ERR_INVALID, "not available with the dense engine");
+  if (!ctx || walker < 0 || walker >= ctx->nw) return fail(ctx, VMC_ERR_INVALID, "bad arguments");
+  if (!ctx->ready) return fail(ctx, VMC_ERR_STATE, "positions not set");
+  Params P;
+  const LaunchCfg L = factor_cfg(ctx, P);
+  P.ilu_wait_ns = 0;
+  CK(launch_refactor(L, ctx->dW, walker, P, 1), "refactor kernel");
+  ctx->pending[walker] = 0;
+  return check_walker_status(ctx);
 }
 
 extern "C" vmc_status vmc_philox_device(const uint32_t* ctr, const uint32_t* key, uint32_t* out, int n) {

@@ -179,6 +179,7 @@ struct Params {
   int warp_rows;    // levels of at most this many rows: triangular-solve rows by one warp, no barrier
   int tri_group;    // > 1: blocked triangular solves, blocks of 8 x this many rows
   int lane_entries; // entries per lane the triangular solves' lane groups are sized for
+  unsigned long long ilu_wait_ns;  // longest wait of an ILUTP row for the row before it (vmc_ilutp.cuh)
   // budgeted advance of the persistent engine: the walkers claim moves one at a time from
   // *budget_ctr until budget_total are claimed (nullptr: fixed sweeps)
   unsigned long long* budget_ctr;
@@ -390,6 +391,9 @@ __device__ __forceinline__ void st_release(int* p, int v) {
   asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 __device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+// Longest wait of an ILUTP row for the row before it, in ns (Params::ilu_wait_ns; a row takes
+// about 0.1 ms).
+constexpr unsigned long long kIluWaitNs = 1000000000ull;
 // Longest wait between the two CTAs of a walker pair (either side), in ns.
 constexpr unsigned long long kPairWaitNs = 30ull * 1000000000ull;
 // Wait (thread 0) until *state differs from `from`; returns the new value, or -1 after

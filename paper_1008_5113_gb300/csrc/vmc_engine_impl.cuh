@@ -51,8 +51,12 @@ __device__ __noinline__ void solve_with_controller(const Walker& w, const Params
       if (fl & 2) c->status = ST_CAPACITY;
     }
     __syncthreads();
-    solve_move<T>(w, P, w.row_of_part[k], rtol, 4 * (2 + P.max_restarts), o, sh);  // and allow more cycles
-    flush_counts<T>(w, sh);
+    if (fl & 4) {
+      o.status = ST_TIMEOUT;  // no factors to solve with; the status is set
+    } else {
+      solve_move<T>(w, P, w.row_of_part[k], rtol, 4 * (2 + P.max_restarts), o, sh);  // and allow more cycles
+      flush_counts<T>(w, sh);
+    }
   }
   const int kits = o.its_trig >= 0 ? o.its_trig : o.total_its;  // iterations to the tolerance
   int cause = 0;
@@ -170,7 +174,7 @@ __device__ __noinline__ void commit_move(const Walker& w, const Params& P, int k
   } else {
     int fl = factor_block<T>(w, P, sh, false);
     if (tid == 0) c->refactors_updates += 1;
-    if (fl & 1) {
+    if ((fl & 5) == 1) {
       fl = factor_block<T>(w, P, sh, true);
       if (tid == 0) { c->reorders += 1; c->reorder_breakdown += 1; }
     }
@@ -451,7 +455,7 @@ __device__ __noinline__ void af_factor_loop(const Walker& w0, const Params& P, i
     const int fl = factor_block<T>(wf, P, sh, P.af_reorder != 0);
     __syncthreads();
     if (threadIdx.x == 0) {
-      c->af_fail = fl & 3;
+      c->af_fail = (fl & 3) | (fl >> 2 & 1);  // a wait that ran out: the solver factors again itself
       __threadfence();
       st_release(&c->af_state, 2);
     }

@@ -59,7 +59,10 @@ __device__ __forceinline__ PipePlan ilu_pipe_plan(int n, size_t dbytes, int nwar
 
 // Block-wide; the first pl.warps warps factor.  over: global scratch for the values beyond
 // kPipeVals, kMaxRowNZ - kPipeVals per warp (needed when n > kPipeVals).  Results as
-// ilutp_warp (thread 0 has them), except the L levels, which the caller computes.
+// ilutp_warp (thread 0 has them), except the L levels, which the caller computes.  Bit 2 of the
+// result: a wait ran out (P.ilu_wait_ns) and the rows are incomplete -- the column permutation
+// is one, but unfinished rows hold the entries of an older factorisation, in its labels, so
+// nothing may be built from them.
 template <typename W>
 __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared& sh, const PipePlan& pl, W* over_all,
                                        int* npiv_out, double* nnz_out, int* p_out) {
@@ -182,7 +185,7 @@ __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared&
             const unsigned long long t0 = global_ns();
             while ((d2 = *done) == d && !*lost) {
               __nanosleep(20);
-              if (global_ns() - t0 > 1000000000ull) *lost = 1;
+              if (global_ns() - t0 > P.ilu_wait_ns) *lost = 1;
             }
           }
           d2 = __shfl_sync(0xffffffffu, d2, 0);
@@ -393,15 +396,12 @@ __device__ __noinline__ int ilutp_pipe(const Walker& w, const Params& P, Shared&
     w.perm[i] = perm[i];
     w.iperm[i] = ip[i];
   }
-  if (threadIdx.x == 0) {
-    w.ctl->ilu_rows += n;
-    if (sh.ilu_lost) sh.iflag[3] = 1;  // a wait ran out: reported as VMC_ERR_TIMEOUT
-  }
+  if (threadIdx.x == 0) w.ctl->ilu_rows += n;
   __syncthreads();
   *npiv_out = sh.ilu_npiv;
   *nnz_out = (double)sh.ilu_nnz;
   *p_out = p;
-  return sh.ilu_flags | (sh.ilu_lost ? 1 : 0);
+  return sh.ilu_flags | (sh.ilu_lost ? 4 : 0);
 }
 
 }  // namespace vmc

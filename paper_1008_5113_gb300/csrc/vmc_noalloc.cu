@@ -237,6 +237,7 @@ extern "C" vmc_status vmc_ratio_noalloc(const vmc_system* sys, const vmc_solver_
   P.tri_group = p.trisolve == 1 ? 1 : std::min(std::max(p.trisolve_group, 1), 64);
   P.lane_entries = p.trisolve_lane_entries > 0 ? std::min(p.trisolve_lane_entries, 64) : (fp64 ? 8 : 2);
   P.step_limit = 0;
+  P.ilu_wait_ns = kIluWaitNs;
   // shared-memory plan for a single walker CTA
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);

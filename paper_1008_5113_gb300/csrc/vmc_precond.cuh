@@ -1108,7 +1108,9 @@ __device__ __noinline__ void relabel_and_levels(const Walker& w, const Params& P
 }
 
 // Full (re)factorisation: optional reorder, ILUTP, levels; clears the update chain.
-// Block-wide.  Returns the ILUTP flags.
+// Block-wide.  Returns the ILUTP flags.  A wait that ran out (bit 2) is recorded in the walker's
+// status here, whatever launch it happens in, and the streams stay those of the factorisation
+// before: levels and streams of incomplete rows would index out of their arrays.
 template <typename T>
 __device__ __noinline__ int factor_block(const Walker& w, const Params& P, Shared& sh, bool reorder) {
   const long long t0 = clock64();
@@ -1153,12 +1155,14 @@ __device__ __noinline__ int factor_block(const Walker& w, const Params& P, Share
       c->n_upd = 0;
       c->upd_nnz = 0;
       c->last_breakdown = fl & 1;
-      c->fresh = reorder ? 1 : 0;  // a synchronous reorder + refactorisation of the current matrix
+      c->fresh = reorder && !(fl & 4) ? 1 : 0;  // a synchronous reorder + refactorisation of the current matrix
+      if ((fl & 4) && c->status == ST_OK) c->status = ST_TIMEOUT;
       c->af_epoch += 1;  // a background factorisation requested before this one is stale
     }
   }
   __syncthreads();
   fl = sh.iflag[0];
+  if (fl & 4) return fl;  // the same in every thread
   const long long tl = clock64();
   relabel_and_levels<T>(w, P, sh);
   if (threadIdx.x == 0) w.ctl->cyc[PH_LEVELS] += clock64() - tl;

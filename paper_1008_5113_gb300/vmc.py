@@ -106,6 +106,7 @@ _SIG = {
     "vmc_philox_device": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_int]),
     "vmc_kernel_bench": (C.c_int, [C.c_void_p, C.c_int, C.c_int]),
     "vmc_check_wait_timeout": (C.c_int, [C.c_void_p]),
+    "vmc_check_factor_timeout": (C.c_int, [C.c_void_p, C.c_int]),
     "vmc_ratio_noalloc": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_int, C.c_void_p, C.c_void_p,
                                     C.c_void_p]),
     "vmc_noalloc_capacity": (C.c_size_t, []),
@@ -336,6 +337,11 @@ def vmc_kernel_bench(ctx, which: int, reps: int) -> None:
 def vmc_check_wait_timeout(ctx) -> int:
     """Status of the bounded-wait check (VMC_ERR_TIMEOUT = 6 expected)."""
     return lib().vmc_check_wait_timeout(ctx)
+
+
+def vmc_check_factor_timeout(ctx, walker: int) -> int:
+    """Status of a refactorisation whose waits run out (VMC_ERR_TIMEOUT = 6 expected)."""
+    return lib().vmc_check_factor_timeout(ctx, walker)
 
 
 def vmc_philox_device(ctr, key) -> np.ndarray:
