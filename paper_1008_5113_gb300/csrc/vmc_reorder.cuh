@@ -13,9 +13,13 @@
 // warp searches the lattice cells around the particle (orbitals are sites; particles are
 // kept in a list per cell) out to a radius that holds the nearest one for certain, and scans
 // the positions only when few are left or nothing near is free.  Distances are compared in
-// FP32 first; FP64 decides between those that FP32 cannot tell apart, so the result is the
-// rule's.  Measured, one walker's reordering: n = 1000 12.4 -> 2.1 ms, n = 4096 214 -> 13 ms
-// (397 ms where two CTAs shared an SM).
+// FP32 first, in units of the lattice constant, from a copy of the coordinates made for it (any
+// constant gives the same comparisons, and a search converts nothing); FP64 decides between
+// those that FP32 cannot tell apart, so the result is the rule's.  Positions outside the box,
+// which the FP32 minimum image and the cells do not cover, are scanned in FP64.  Measured, one walker's reordering: n = 1000 12.4 -> 2.1 ms, n = 4096
+// 214 -> 13 ms (397 ms where two CTAs shared an SM) with the coordinates converted in every
+// search; the copy takes n = 1000 from 3.05 to 2.37 ms and n = 4096 from 13.9 to 11.0 ms
+// (electrons 0.2 a from their sites).
 #pragma once
 #include "vmc_geom.cuh"
 
@@ -29,13 +33,16 @@ struct Nearest {
 
 // Nearest candidate of a warp's search: each(f) calls f(position, FP32 distance^2, id) for
 // the lane's candidates, exact(id) is the FP64 distance^2.  limit: FP32 distances^2 at or
-// beyond it do not count as found (a candidate outside the searched cells may be nearer).
-// margin(d): twice the error of FP32 distances^2 around d.  Returns the position, or -1.
+// beyond it do not count as found (a candidate outside the searched cells may be nearer);
+// kScan: every candidate is among those searched.  margin(d): twice the error of FP32
+// distances^2 around d (infinite: FP64 decides alone).  Returns the position, or -1 (in a scan
+// only when no distance is a number).
+constexpr float kScan = 3e38f;
 template <typename Each, typename Exact, typename Margin>
 __device__ __forceinline__ int nearest_warp(float limit, Each each, Exact exact, Margin margin) {
   float m = 3e38f, thr = 0.0f;
   int cnt = 0, pos = 0x7fffffff;
-  Nearest b{1e300, 0x7fffffff};
+  Nearest b{__longlong_as_double(0x7ff0000000000000ll), 0x7fffffff};
 #pragma unroll 1
   for (int pass = 0; pass < 3; ++pass) {  // the least FP32 distance; who is near it; FP64 among those
     each([&](int p, float d, int id) {
@@ -54,7 +61,7 @@ __device__ __forceinline__ int nearest_warp(float limit, Each each, Exact exact,
     if (pass == 0) {
       m = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(m)));  // d >= 0
       thr = m + margin(m);
-      if (!(thr < limit)) return -1;
+      if (limit < kScan && !(thr < limit)) return -1;
     } else if (pass == 1) {
       if (__reduce_add_sync(0xffffffffu, cnt) == 1) return __reduce_min_sync(0xffffffffu, pos);
     }
@@ -65,7 +72,7 @@ __device__ __forceinline__ int nearest_warp(float limit, Each each, Exact exact,
     const int p2 = __shfl_xor_sync(0xffffffffu, b.pos, o);
     if (d2 < b.d || (d2 == b.d && p2 < b.pos)) { b.d = d2; b.pos = p2; }
   }
-  return b.pos;
+  return b.pos == 0x7fffffff ? -1 : b.pos;
 }
 
 // I: index type of the position tables (16 bits in shared memory, int in global memory).
@@ -74,10 +81,20 @@ __device__ __noinline__ void reorder_search(const Walker& w, I* pos_orb, I* pos_
                                             int* head) {
   const int n = w.n, K = w.K, per = w.per, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
   constexpr int kNone = sizeof(I) == 2 ? 0xffff : -1;
-  // in FP32: a particle within 3e-5 a of a face may be taken for its neighbour cell's, which
-  // the factor 0.9999 on the search limits covers (K <= 64)
-  const float inva = 1.0f / (float)w.a;
-  auto cell_axis = [&](float x) { return min(K - 1, max(0, (int)floorf(x * inva))); };
+  // lengths in units of the lattice constant, FP32: a particle within 3e-5 of a face may be taken
+  // for its neighbour cell's, which the factor 0.9999 on the search limits covers (K <= 64)
+  float* xs = (float*)w.ex_val;  // scratch of at least 8 n doubles, free until the factorisation
+  auto cell_axis = [&](float x) { return min(K - 1, max(0, (int)floorf(x))); };
+  int inside = 1;
+  {
+    const double inva = 1.0 / w.a, L = w.L;
+#pragma unroll 1
+    for (int i = tid; i < 3 * n; i += nt) {
+      const double r = w.R[i];
+      xs[i] = (float)(r * inva);
+      inside &= r >= 0.0 && r < L;
+    }
+  }
 #pragma unroll 1
   for (int c = tid; c < n; c += nt) {
     const int p = w.part_of_row[c], o = w.orb_of_col[c];
@@ -88,19 +105,19 @@ __device__ __noinline__ void reorder_search(const Walker& w, I* pos_orb, I* pos_
   }
 #pragma unroll 1
   for (int c = tid; c < K * K * K; c += nt) head[c] = kNone;
-  __syncthreads();
+  inside = __syncthreads_and(inside);
 #pragma unroll 1
   for (int p = tid; p < n; p += nt) {
-    const double* r = w.R + 3 * p;
-    const int c = cell_axis((float)r[0]) + K * (cell_axis((float)r[1]) + K * cell_axis((float)r[2]));
+    const float* r = xs + 3 * p;
+    const int c = cell_axis(r[0]) + K * (cell_axis(r[1]) + K * cell_axis(r[2]));
     next[p] = (I)atomicExch(&head[c], p);
   }
   __syncthreads();
   if (tid < 32) {
-    const float L = (float)w.L, hL = 0.5f * L, a = (float)w.a;
+    const float L = (float)K, hL = 0.5f * L;
     // coordinates up to L, their differences and the image shift: below 4 x 2^-24 L each,
     // 7 x 2^-24 L on the distance; twice that, times two distances, with room
-    const float eps = 32.0f * 5.9604645e-8f * L;
+    const float eps = inside ? 32.0f * 5.9604645e-8f * L : __int_as_float(0x7f800000);
     auto margin = [&](float d2) { return eps * (1.0f + d2); };  // 2 d <= 1 + d^2
     auto dist32 = [&](float x, float y, float z) {
       x = fabsf(x); y = fabsf(y); z = fabsf(z);
@@ -115,17 +132,17 @@ __device__ __noinline__ void reorder_search(const Walker& w, I* pos_orb, I* pos_
       const float off = 0.5f * (float)b;
       const int cx = c % K;
       c /= K;
-      x = a * ((float)cx + off);
-      y = a * ((float)(c % K) + off);
-      z = a * ((float)(c / K) + off);
+      x = (float)cx + off;
+      y = (float)(c % K) + off;
+      z = (float)(c / K) + off;
     };
     auto wrap_cell = [&](int c) { return c < 0 ? c + K : (c >= K ? c - K : c); };
 #pragma unroll 1
     for (int i = 0; i < n - 1; ++i) {
       const int p = part_at[i];
       const double rp[3] = {w.R[3 * p], w.R[3 * p + 1], w.R[3 * p + 2]};
-      const float px = (float)rp[0], py = (float)rp[1], pz = (float)rp[2];
-      const bool few = n - i <= 64;
+      const float px = xs[3 * p], py = xs[3 * p + 1], pz = xs[3 * p + 2];
+      const bool few = n - i <= 64 || !inside;
       int bj = -1;
       if (!few) {
         const int cx = cell_axis(px), cy = cell_axis(py), cz = cell_axis(pz);
@@ -144,11 +161,11 @@ __device__ __noinline__ void reorder_search(const Walker& w, I* pos_orb, I* pos_
               const int j = (int)pos_orb[o];
               if (j < i) continue;
               const float off = 0.5f * (float)b;
-              f(j, dist32(px - a * ((float)x + off), py - a * ((float)y + off), pz - a * ((float)z + off)), o);
+              f(j, dist32(px - ((float)x + off), py - ((float)y + off), pz - ((float)z + off)), o);
             }
           };
-          // every site outside the searched cells is at least rad * a away along one axis
-          bj = nearest_warp((float)(rad * rad) * a * a * 0.9999f, each,
+          // every site outside the searched cells is at least rad away along one axis
+          bj = nearest_warp((float)(rad * rad) * 0.9999f, each,
                             [&](int o) { return dist2(rp, w.Z + 3 * o, w.L); }, margin);
         }
       }
@@ -162,7 +179,8 @@ __device__ __noinline__ void reorder_search(const Walker& w, I* pos_orb, I* pos_
             f(j, dist32(px - x, py - y, pz - z), o);
           }
         };
-        bj = nearest_warp(3e38f, each, [&](int o) { return dist2(rp, w.Z + 3 * o, w.L); }, margin);
+        bj = nearest_warp(kScan, each, [&](int o) { return dist2(rp, w.Z + 3 * o, w.L); }, margin);
+        if (bj < 0) bj = i;
       }
       if (bj != i) {
         __syncwarp();
@@ -179,8 +197,8 @@ __device__ __noinline__ void reorder_search(const Walker& w, I* pos_orb, I* pos_
       float ox, oy, oz;
       site32(o, ox, oy, oz);
       auto part_dist = [&](int q) {
-        const double* r = w.R + 3 * q;
-        return dist32((float)r[0] - ox, (float)r[1] - oy, (float)r[2] - oz);
+        const float* r = xs + 3 * q;
+        return dist32(r[0] - ox, r[1] - oy, r[2] - oz);
       };
       auto exact = [&](int q) { return dist2(w.R + 3 * q, zo, w.L); };
       int bk = -1;
@@ -207,8 +225,8 @@ __device__ __noinline__ void reorder_search(const Walker& w, I* pos_orb, I* pos_
             }
           };
           // a site lies in [0, 1) of its cell on each axis: cells out to rad hold everything
-          // nearer than rad * a
-          bk = nearest_warp((float)(rad * rad) * a * a * 0.9999f, each, exact, margin);
+          // nearer than rad
+          bk = nearest_warp((float)(rad * rad) * 0.9999f, each, exact, margin);
         }
       }
       if (bk < 0) {
@@ -219,7 +237,8 @@ __device__ __noinline__ void reorder_search(const Walker& w, I* pos_orb, I* pos_
             f(k, part_dist(q), q);
           }
         };
-        bk = nearest_warp(3e38f, each, exact, margin);
+        bk = nearest_warp(kScan, each, exact, margin);
+        if (bk < 0) bk = i;
       }
       __syncwarp();
       if (bk != i && lane == 0) {
