@@ -302,10 +302,14 @@ __device__ void af_swap(const Walker& w0, const Params& P, Shared& sh) {
     for (int j = t0 + 1 + tid; j < len; j += nt) Gi[(size_t)t0 * kMaxUpd + j] = Gi[(size_t)(s0 + t0) * kMaxUpd + s0 + j];
     __syncthreads();
   }
-  int ul = 0;
-  if (tid < len) ul = w0.upd_ulen[s0 + tid];
+  // (single-move calls between two launches may have made the chain longer than the CTA)
+  int* ul = reinterpret_cast<int*>(sh.cpart);
+  static_assert(sizeof(sh.cpart) >= kMaxUpd * sizeof(int), "a length per update");
+#pragma unroll 1
+  for (int j = tid; j < len; j += nt) ul[j] = w0.upd_ulen[s0 + j];
   __syncthreads();
-  if (tid < len) w0.upd_ulen[tid] = ul;
+#pragma unroll 1
+  for (int j = tid; j < len; j += nt) w0.upd_ulen[j] = ul[j];
   if (P.af_reorder) {
     // the new row pairing comes with the factors; the chain lives in column space and
     // x = A_p^{-1} e_{row(k)} does not depend on the row order, so it carries over
