@@ -422,7 +422,7 @@ static int dense_cluster(int nwalk, int max_n, int static_smem) {
 template <typename K, typename... A>
 static cudaError_t dense_launch(K kernel, const LaunchCfg& L, int nwalk, int max_n, A... args) {
   cudaFuncAttributes fa{};
-  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+  const cudaError_t e = allow_dynamic_smem(kernel, &fa);
   if (e != cudaSuccess) return e;
   const int cs = dense_cluster(nwalk, max_n, (int)fa.sharedSizeBytes);
   cudaLaunchConfig_t lc = {};
@@ -437,10 +437,6 @@ static cudaError_t dense_launch(K kernel, const LaunchCfg& L, int nwalk, int max
   at[0].val.clusterDim.z = 1;
   lc.attrs = at;
   lc.numAttrs = cs > 1 ? 1 : 0;
-  if (lc.dynamicSmemBytes + fa.sharedSizeBytes > 48 * 1024) {
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lc.dynamicSmemBytes);
-    if (e != cudaSuccess) return e;
-  }
   return cudaLaunchKernelEx(&lc, kernel, args..., cs);
 }
 

@@ -824,14 +824,9 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_bench(const Walker* __restri
 // ---------------------------------------------------------------------------
 // templated host launchers (one instantiation per working precision)
 // ---------------------------------------------------------------------------
-template <typename K>
-static cudaError_t prep(K kernel, const LaunchCfg& L) {
-  if (L.smem > 48 * 1024) return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
-  return cudaSuccess;
-}
 #define VMC_LAUNCH(KERNEL, GRID, ...)                                   \
   do {                                                                 \
-    cudaError_t e_ = prep(KERNEL, L);                                  \
+    cudaError_t e_ = allow_dynamic_smem(KERNEL);                       \
     if (e_ != cudaSuccess) return e_;                                  \
     KERNEL<<<(GRID), L.threads, L.smem, L.stream>>>(__VA_ARGS__);      \
     return cudaGetLastError();                                         \
@@ -871,12 +866,14 @@ cudaError_t launch_sweep_pair_T(const LaunchCfg& L, const Walker* W, int walker0
   at[0].val.clusterDim.z = 1;
   lc.attrs = at;
   lc.numAttrs = 1;
-  cudaError_t e = prep(k_sweep_pair<T, kPerSm>, L);
+  cudaError_t e = allow_dynamic_smem(k_sweep_pair<T, kPerSm>);
   if (e != cudaSuccess) return e;
   return cudaLaunchKernelEx(&lc, k_sweep_pair<T, kPerSm>, W, walker0, P, n_sweeps, sweep0, sigma, seeds, acc, ratio, launch_id);
 }
 template <typename T>
-cudaError_t prepare_step_kernels_T(const LaunchCfg& L) { return L.per_sm > 1 ? prep(k_step<T, 2>, L) : prep(k_step<T, 1>, L); }
+cudaError_t prepare_step_kernels_T(const LaunchCfg& L) {
+  return L.per_sm > 1 ? allow_dynamic_smem(k_step<T, 2>) : allow_dynamic_smem(k_step<T, 1>);
+}
 template <typename T>
 cudaError_t launch_step_T(const LaunchCfg& L, const Walker* W, int walker0, int nwalk, const Params& P, int q,
                           int n_sweeps, int s_local, long long sweep0, double sigma, const uint64_t* seeds,

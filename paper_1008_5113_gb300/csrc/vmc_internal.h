@@ -17,6 +17,21 @@ struct LaunchCfg {
   size_t smem;  // dynamic shared memory per walker CTA
   int per_sm;   // walker CTAs an SM is to hold (1 or 2)
 };
+// Lets a kernel be launched with any dynamic shared memory that the device has beside its static
+// one.  Always the same value: contexts of different sizes may launch the kernel from several
+// threads, and a context's own size, set before its launch, could be lowered by another's in
+// between ("too many resources requested for launch").  About 1 us of host time.
+template <typename K>
+cudaError_t allow_dynamic_smem(K kernel, cudaFuncAttributes* attributes = nullptr) {
+  cudaFuncAttributes fa{};
+  int dev = 0, optin = 0;
+  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (attributes) *attributes = fa;
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+}
 // static shared memory of the walker kernels (bytes)
 int kernel_static_smem(bool fp64);
 
