@@ -509,8 +509,8 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     o.push_back(cv.take<int>(n));                      // 31 gP
     o.push_back(cv.take<int>(n));                      // 32 gQ
     o.push_back(cv.take<char>((size_t)mu * ld * Tsz)); // 33 upd_z
-    o.push_back(cv.take<int>((size_t)kMaxUpd * kMaxU));     // 34 upd_ucol
-    o.push_back(cv.take<char>((size_t)kMaxUpd * kMaxU * Tsz));  // 35 upd_uval
+    o.push_back(cv.take<int>((size_t)mu * kMaxU));     // 34 upd_ucol
+    o.push_back(cv.take<char>((size_t)mu * kMaxU * Tsz));  // 35 upd_uval
     o.push_back(cv.take<int>(mu));                     // 36 upd_ulen
     o.push_back(cv.take<double>((size_t)kMaxUpd * kMaxUpd));  // 37 upd_G
     o.push_back(cv.take<char>((size_t)(m + 1) * ld * Tsz));   // 38 V

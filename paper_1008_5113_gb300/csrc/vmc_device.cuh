@@ -134,6 +134,7 @@ struct Walker {
   int* lev_l; int* lev_u;
   int* l_lvl_ptr; int* l_lvl_rows; int* u_lvl_ptr; int* u_lvl_rows; int* lvl_cur;
   double* wrow; int* wpos; int* gP; int* gQ;
+  // update chain: rows of z_hat; entry t of u_s at t mu + s (mu x kMaxU of them); lengths; inverse
   void* upd_z; int* upd_ucol; void* upd_uval; int* upd_ulen; double* upd_G;
   void* V; void* Zk; void* tv;
   double* x64; double* r64;

@@ -142,8 +142,8 @@ __device__ __noinline__ void commit_move(const Walker& w, const Params& P, int k
     for (int i = tid; i < n; i += nt) zs[i] = (T)(w.x64[i] * inv);
 #pragma unroll 1
     for (int t = tid; t < ulen; t += nt) {  // the update index fastest: see update_chain
-      w.upd_ucol[(size_t)t * kMaxUpd + s] = sh.ucol[t];
-      Uv[(size_t)t * kMaxUpd + s] = (T)sh.uval[t];
+      w.upd_ucol[t * w.mu + s] = sh.ucol[t];
+      Uv[t * w.mu + s] = (T)sh.uval[t];
     }
     if (tid == 0) { w.upd_ulen[s] = ulen; c->upd_nnz += ulen; }
     __syncthreads();
@@ -285,8 +285,8 @@ __device__ void af_swap(const Walker& w0, const Params& P, Shared& sh) {
   T* Uv = (T*)w0.upd_uval;
 #pragma unroll 1
   for (int t = tid; t < kMaxU; t += nt) {
-    int* uc = w0.upd_ucol + (size_t)t * kMaxUpd;
-    T* uu = Uv + (size_t)t * kMaxUpd;
+    int* uc = w0.upd_ucol + (size_t)t * w0.mu;
+    T* uu = Uv + (size_t)t * w0.mu;
 #pragma unroll 1
     for (int j = 0; j < len; ++j)
       if (t < w0.upd_ulen[s0 + j]) {

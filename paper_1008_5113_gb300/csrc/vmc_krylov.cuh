@@ -509,7 +509,7 @@ __device__ __forceinline__ const T* tri_both(const Walker& w, const Params& P, c
 template <typename T>
 __device__ __forceinline__ void update_chain(const Walker& w, T* zs, T* zout, Shared& sh) {
   const int n = w.n, tid = threadIdx.x, nt = blockDim.x, mu = w.ctl->n_upd;
-  const int ld = w.ld;
+  const int ld = w.ld, lu = w.mu;
   if (mu == 0) {
     if (zout != zs) {
 #pragma unroll 1
@@ -532,7 +532,7 @@ __device__ __forceinline__ void update_chain(const Walker& w, T* zs, T* zout, Sh
           const T* uu = (const T*)w.upd_uval + s;
           const int* uc = w.upd_ucol + s;
 #pragma unroll 4
-          for (int t = g; t < ul; t += G) acc += (double)uu[(size_t)t * kMaxUpd] * (double)zs[uc[(size_t)t * kMaxUpd]];
+          for (int t = g; t < ul; t += G) acc += (double)uu[t * lu] * (double)zs[uc[t * lu]];
         } else {
           const double* gi = w.upd_G + s;
           if (g == 0) acc = sh.cupd[s];
