@@ -339,6 +339,8 @@ __device__ void af_swap(const Walker& w0, const Params& P, Shared& sh) {
     st_release(&c->af_state, 0);
   }
   fence_proxy_async_global();  // the new streams are read by bulk copies next
+  // ... into the ring, which task streams, if the old set had them, used with plain accesses
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
 }
 
