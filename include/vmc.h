@@ -138,8 +138,8 @@ typedef struct {
                           flight on several warps of the CTA where the working rows of at least
                           two fit its shared memory; else one warp, with the working row as a
                           hash map keyed by label when the dense working row of n entries does
-                          not fit the shared memory (and n <= 65535), else the dense row; 1 = as
-                          0, but never the hash map; 2 = always the hash map where it fits (0) */
+                          not fit the shared memory (and n <= 65535), else the dense row; 1 =
+                          always the dense row; 2 = always the hash map where it fits (0) */
   int trisolve_warp_rows; /* level-by-level triangular solves from the chunk streams: a level of at most this many
                           rows, <= 32, is solved by one warp alone, with no barrier among the
                           solving warps after it (the other warps meet it before the next larger

@@ -176,7 +176,7 @@ struct Params {
   int y_half;       // byte offset of the second solve vector (tri_sf)
   double trig_rtol; // controller: the solve converged if its residual reached this ...
   int trig_its;     // ... within this many GMRES iterations (all cycles)
-  int ilu_variant;  // 0: auto (hash working row where the dense one misses shared memory); 1: dense; 2: hash
+  int ilu_variant;  // 0: auto (rows in flight, else one warp by size); 1: one warp, dense row; 2: one warp, hashed row
   int warp_rows;    // levels of at most this many rows: triangular-solve rows by one warp, no barrier
   int tri_group;    // > 1: blocked triangular solves, blocks of 8 x this many rows
   int lane_entries; // entries per lane the triangular solves' lane groups are sized for

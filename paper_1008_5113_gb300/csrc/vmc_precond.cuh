@@ -1122,11 +1122,11 @@ __device__ __noinline__ int factor_block(const Walker& w, const Params& P, Share
   int npiv = 0, p = 0, fl = 0;
   double nnz = 0.0;
   // rows in flight on several warps where at least two warps' working rows fit shared memory;
-  // else one warp: the hashed working row where the dense one does not fit shared memory
-  // (n > 6000 or so, or forced), else the dense row
+  // else, or when a variant is asked for, one warp: the hashed working row where the dense one
+  // does not fit shared memory (n > 6000 or so, or asked for), else the dense row
   const PipePlan pp = P.ilu64 ? ilu_pipe_plan<double>(w.n, (size_t)P.dsm_bytes, blockDim.x >> 5)
                               : ilu_pipe_plan<T>(w.n, (size_t)P.dsm_bytes, blockDim.x >> 5);
-  if (pp.warps >= 2 && P.ilu_variant != 2 && w.ex_val != nullptr && w.u_head != nullptr) {
+  if (pp.warps >= 2 && P.ilu_variant == 0 && w.ex_val != nullptr && w.u_head != nullptr) {
     fl = P.ilu64 ? ilutp_pipe<double>(w, P, sh, pp, w.ex_val, &npiv, &nnz, &p)
                  : ilutp_pipe<T>(w, P, sh, pp, (T*)w.ex_val, &npiv, &nnz, &p);
   } else if (threadIdx.x < 32) {

@@ -58,3 +58,22 @@ def test_lost_factorisation_is_reported(vmc, prec, kw):
         assert np.all(np.isfinite(rat))
     finally:
         vmc.vmc_destroy(ctx)
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2])
+@pytest.mark.parametrize("K,lat,kw", [(6, 0, {}), (11, 0, dict(lfil_extra=16)), (5, 1, dict(block_threads=64))])
+def test_ilutp_variants(vmc, prec, K, lat, kw):
+    """Variants 1 and 2 have one row in flight, so no wait that could run out; their factors are
+    those of the rows in flight, bit for bit."""
+    sysd = (K, 0, 1.0, 2.0, 1.45) if lat == 0 else (K, 1, 2.031, 1.0, 3.39)
+    R = O.initial_positions(O.system(*sysd), 5, 0.25 * sysd[2])
+    out = []
+    for variant, status in ((0, 6), (1, 0), (2, 0)):
+        ctx = vmc.vmc_create([sysd], vmc.params(precision=prec, ilutp_variant=variant, **kw))
+        try:
+            vmc.vmc_set_positions(ctx, 0, R)
+            out.append([x.tobytes() for x in vmc.vmc_get_factors(ctx, 0)])
+            assert vmc.vmc_check_factor_timeout(ctx, 0) == status
+        finally:
+            vmc.vmc_destroy(ctx)
+    assert out[0] == out[1] == out[2]
