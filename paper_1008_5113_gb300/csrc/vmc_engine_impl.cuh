@@ -811,7 +811,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_bench(const Walker* __restri
         __syncthreads();
         spmv<T>(w, z_ring<T>(P), (const T*)nullptr, (T*)dyn_smem());
       } else {
-        spmv<T>(w, V, (const T*)nullptr, Zk);
+        spmv<T>(w, stage_x<T>(w, P, V), (const T*)nullptr, Zk);
       }
       if (threadIdx.x == 0) w.ctl->alg_bytes += w.ctl->nnz_A * (sizeof(T) + 4) + (double)n * (2 * sizeof(T) + 4);
     } else {

@@ -176,6 +176,21 @@ __device__ __forceinline__ void spmv(const Walker& w, const T* x, const T* v, T*
   }
 }
 
+// The product's input vector copied into the solve area where that is in shared memory (idle
+// between preconditioner applies): the gathers then read shared memory instead of scattered
+// global lines.  For walkers whose vectors the task ring does not hold (FP32 from n = 24 000 or
+// so, FP64 from 12 000) and for the chunk streams.  n = 32768 x 152 walkers FP32: an apply 449 us
+// gathering from global memory, 283 us so (kappa 1, r_c 2: 644, 406).
+// Block-wide, ends synchronised; returns the vector to read.
+template <typename T>
+__device__ __forceinline__ const T* stage_x(const Walker& w, const Params& P, const T* x) {
+  if (!P.y_smem) return x;
+  T* xs = (T*)dyn_smem();
+  block_copy(xs, x, w.n);
+  __syncthreads();
+  return xs;
+}
+
 // Shared-memory ring of the stream chunks: one mbarrier per slot, initialised once
 // per kernel launch; chunk g of the launch lives in slot g % S, phase (g / S) & 1.
 __device__ __forceinline__ void ring_init(Shared& sh, const Params& P) {
@@ -752,7 +767,7 @@ __device__ __forceinline__ int gmres_cycle(const Walker& w, const Params& P, dou
     // the vector that joins the basis is A M v - v: the same Krylov space, and with a good
     // preconditioner A M v is mostly v, whose removal by projection alone would cancel nearly
     // all of w and need the second Gram-Schmidt pass every time; ||A M v - v|| is the monitor
-    spmv<T>(w, SM ? z_ring<T>(P) : zj, vj, wv);
+    spmv<T>(w, SM ? z_ring<T>(P) : stage_x<T>(w, P, zj), vj, wv);
     if (tid < ld - n) wv[n + tid] = (T)0;
     __syncthreads();
     const long long to = clock64();
