@@ -113,66 +113,105 @@ __device__ __forceinline__ const float* ell_vals<float>(const Walker& w) { retur
 template <>
 __device__ __forceinline__ const double* ell_vals<double>(const Walker& w) { return w.ell_val; }
 
+// Loads that are issued where they stand (see Wide).
+__device__ __forceinline__ int load_now(const int* p) {
+  int v;
+  asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float load_now(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double load_now(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+
 // 16-bit columns and values of four entries of a row in the transposed copy.
 template <typename T>
 struct EllQuad {
   unsigned c0, c1;  // two columns each
   Wide<T> v[sizeof(T) / 4];
-  __device__ __forceinline__ void load(const unsigned short* col, const T* val, size_t at) {
-    asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(c0), "=r"(c1) : "l"(col + at));
+  __device__ __forceinline__ void load(const unsigned short* col, const T* val) {
+    asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(c0), "=r"(c1) : "l"(col));
 #pragma unroll
-    for (int k = 0; k < (int)sizeof(T) / 4; ++k) v[k].load(val + at + kWide<T> * k);
+    for (int k = 0; k < (int)sizeof(T) / 4; ++k) v[k].load(val + kWide<T> * k);
   }
   __device__ __forceinline__ T value(int u) const { return v[u / kWide<T>].v[u % kWide<T>]; }
 };
 
-// Dot product of particle p's row with x.  From the transposed copy of the slots (quads of
+// Dot product of particle p's row (len entries) with x.  From the transposed copy of the slots (quads of
 // entries, quad q of every particle side by side, zeros past the row's end): coalesced
 // 8- and 16-byte loads, all of a row of up to 24 entries in flight, summed in entry order;
-// else from the slot itself.
+// else from the slot itself.  Two running pointers: as twelve precomputed addresses they made
+// the solve spill around the loads (in an iteration of 256 walkers of n = 4096, two an SM, FP32:
+// product 63.9 us, FP64 residual 53.7; so 55.2 and 43.1; with five quads in flight 41.2 and 55.0,
+// but a second trip for the rows beyond 20 entries: one walker of n = 4096 14.3 us, 12.0 so).
 template <typename T, typename X>
-__device__ __forceinline__ X row_dot(const Walker& w, int p, const X* x) {
-  const int cap = w.cap, len = w.a_len[p];
+__device__ __forceinline__ X row_dot(const Walker& w, int p, int len, const X* x) {
+  const int cap = w.cap;
   if (w.ell_col == nullptr) {
     const T* v = sizeof(T) == 4 ? (const T*)w.a_val32 : (const T*)w.a_val;
     return slot_dot<T, X>(w.a_col + (size_t)p * cap, v + (size_t)p * cap, len, cap, x);
   }
-  const unsigned short* col = w.ell_col;
-  const T* val = ell_vals<T>(w);
   const size_t step = 4 * (size_t)w.ld;
+  const unsigned short* col = w.ell_col + 4 * (size_t)p;
+  const T* val = ell_vals<T>(w) + 4 * (size_t)p;
   constexpr int U = 6;
   X acc = 0;
-  size_t at = 4 * (size_t)p;
 #pragma unroll 1
-  for (int t0 = 0; t0 < len; t0 += 4 * U) {
+  for (int left = len; left > 0; left -= 4 * U) {
     EllQuad<T> e[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (t0 + 4 * u < len) e[u].load(col, val, at + u * step);
+    for (int u = 0; u < U; ++u) {
+      if (4 * u < left) e[u].load(col, val);
+      col += step;
+      val += step;
+      asm volatile("" : "+l"(col), "+l"(val));
+    }
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if (t0 + 4 * u < len) {
+      if (4 * u < left) {
         acc += (X)e[u].value(0) * x[e[u].c0 & 0xffffu];
         acc += (X)e[u].value(1) * x[e[u].c0 >> 16];
         acc += (X)e[u].value(2) * x[e[u].c1 & 0xffffu];
         acc += (X)e[u].value(3) * x[e[u].c1 >> 16];
       }
-    at += U * step;
   }
   return acc;
 }
 
+// The length and the row of A_p of the thread's particles, read one particle ahead: a row's
+// entries and v's element then start without a memory round trip before them.
+struct NextRow {
+  int len, row;
+  __device__ __forceinline__ NextRow(const Walker& w, int p) : len(0), row(0) {
+    if (p < w.n) {
+      len = load_now(w.a_len + p);
+      row = load_now(w.row_of_part + p);
+    }
+  }
+};
+
 // y = A_p x - v (v may be null): a particle's row per thread in slot order, the result
-// scattered to its row of A_p.
+// scattered to its row of A_p.  Bound by memory round trips: with a row's length, then its
+// entries, and v's place, then v, one after the other, an apply of 152 walkers of n = 32768 took
+// 283 us in FP32, 64 of n = 8000 88, 64 of n = 1000 10.0 (FP64 14.0); so 216, 43, 4.4 (7.3).
+// (v subtracted in a pass of its own, without the gather: 64 of n = 8000 89 us an iteration's
+// product, 55 with it; n = 216 FP64 3.7 and 3.2.)
 template <typename T>
 __device__ __forceinline__ void spmv(const Walker& w, const T* x, const T* v, T* y) {
   const int n = w.n;
-  const int* rop = w.row_of_part;
+  NextRow at(w, threadIdx.x);
 #pragma unroll 1
   for (int p = threadIdx.x; p < n; p += blockDim.x) {
-    const int r = rop[p];
-    const T vr = v ? v[r] : (T)0;
-    y[r] = row_dot<T, T>(w, p, x) - vr;
+    const NextRow next(w, p + blockDim.x);
+    const T vr = v ? load_now(v + at.row) : (T)0;
+    y[at.row] = row_dot<T, T>(w, p, at.len, x) - vr;
+    at = next;
   }
 }
 
@@ -916,15 +955,17 @@ __device__ __forceinline__ void residual64(const Walker& w, int brow, Shared& sh
   const int n = w.n, nt = blockDim.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
   const long long t0 = clock64();
   double s[3] = {0.0, 0.0, 0.0};
+  NextRow at(w, tid);
 #pragma unroll 1
   for (int p = tid; p < n; p += nt) {  // slots in order (see spmv)
-    const int r = w.row_of_part[p];
-    const double xp = w.x64[p];
-    const double acc = row_dot<double, double>(w, p, w.x64);
-    const double rr = (r == brow ? 1.0 : 0.0) - acc;
-    w.r64[r] = rr;
+    const NextRow next(w, p + nt);
+    const double xp = load_now(w.x64 + p);
+    const double acc = row_dot<double, double>(w, p, at.len, w.x64);
+    const double rr = (at.row == brow ? 1.0 : 0.0) - acc;
+    w.r64[at.row] = rr;
     s[0] += rr * rr;
     s[1] += xp * xp;
+    at = next;
   }
 #pragma unroll 1
   for (int t = tid; t < sh.ulen; t += nt) s[2] += sh.uval[t] * w.x64[sh.ucol[t]];
