@@ -782,9 +782,11 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_apply_precond(const Walker* 
 
 // Microbenchmark: `reps` back-to-back applications of one hot-path kernel per walker
 // (0: L and U triangular solves, 1: SpMV in the working precision, 2: the full
-// preconditioner apply with the update chain), on V[0] = 1 / sqrt(n).
-template <typename T>
-__global__ void __launch_bounds__(kMaxThreads, 2) k_bench(const Walker* __restrict__ W, Params P_, int which, int reps) {
+// preconditioner apply with the update chain), on V[0] = 1 / sqrt(n).  A kernel for each, and
+// for each occupancy of the sweeping kernels: in one kernel of 128 registers all three had the
+// spills of the largest.
+template <typename T, int kPerSm, int kWhich>
+__global__ void __launch_bounds__(kMaxThreads, kPerSm) k_bench(const Walker* __restrict__ W, Params P_, int reps) {
   __shared__ Shared sh;
   const Params& P = stage_params(sh, P_);
   ring_init(sh, P);
@@ -798,21 +800,25 @@ __global__ void __launch_bounds__(kMaxThreads, 2) k_bench(const Walker* __restri
   const bool sm = krylov_in_smem<T>(w, P);
 #pragma unroll 1
   for (int it = 0; it < reps; ++it) {
-    if (which == 0) {
+    if constexpr (kWhich == 0) {
       const long long t0 = clock64();
       const T* y = tri_both<T>(w, P, V, sh);
       if (threadIdx.x == 0) sh.cyc[PH_TRI] += clock64() - t0;
       block_scatter(Zk, w.perm, y, n);
       if (threadIdx.x == 0)
         w.ctl->alg_bytes += w.ctl->nnz_LU * (sizeof(T) + 4) + (double)n * (3 * sizeof(T) + 8);
-    } else if (which == 1) {
+    } else if constexpr (kWhich == 1) {
+      const T* x = V;
+      T* y = Zk;
       if (sm) {  // as in an iteration: the input in the task ring, the result in the solve area
         block_copy(z_ring<T>(P), V, n);
         __syncthreads();
-        spmv<T>(w, z_ring<T>(P), (const T*)nullptr, (T*)dyn_smem());
+        x = z_ring<T>(P);
+        y = (T*)dyn_smem();
       } else {
-        spmv<T>(w, stage_x<T>(w, P, V), (const T*)nullptr, Zk);
+        x = stage_x<T>(w, P, V);
       }
+      spmv<T>(w, x, (const T*)nullptr, y);
       if (threadIdx.x == 0) w.ctl->alg_bytes += w.ctl->nnz_A * (sizeof(T) + 4) + (double)n * (2 * sizeof(T) + 4);
     } else {
       precond_apply<T, false>(w, P, V, Zk, sh);
@@ -909,7 +915,13 @@ cudaError_t launch_apply_precond_T(const LaunchCfg& L, const Walker* W, int wi, 
 }
 template <typename T>
 cudaError_t launch_bench_T(const LaunchCfg& L, const Walker* W, int nwalk, const Params& P, int which, int reps) {
-  VMC_LAUNCH(k_bench<T>, nwalk, W, P, which, reps);
+  const bool two = L.per_sm > 1;
+  if (which == 0 && two) VMC_LAUNCH((k_bench<T, 2, 0>), nwalk, W, P, reps);
+  if (which == 0) VMC_LAUNCH((k_bench<T, 1, 0>), nwalk, W, P, reps);
+  if (which == 1 && two) VMC_LAUNCH((k_bench<T, 2, 1>), nwalk, W, P, reps);
+  if (which == 1) VMC_LAUNCH((k_bench<T, 1, 1>), nwalk, W, P, reps);
+  if (two) VMC_LAUNCH((k_bench<T, 2, 2>), nwalk, W, P, reps);
+  VMC_LAUNCH((k_bench<T, 1, 2>), nwalk, W, P, reps);
 }
 
 }  // namespace vmc
