@@ -74,6 +74,7 @@ void plan_smem(int ybytes, int budget, Params& P, bool allow_sf) {
   P.ring_slots = std::min(kMaxSlots, avail / P.slot_bytes);
   // the rest of the budget is ILUTP scratch (work row, U-row cache)
   P.dsm_bytes = std::max(budget, P.y_bytes + P.ring_slots * P.slot_bytes);
+  P.ring_bytes = (P.dsm_bytes - P.y_bytes) & ~127;
 }
 
 static int count_sites_within(int lattice, double a, double gx, double gy, double gz, double R) {

@@ -167,6 +167,7 @@ struct Params {
   int y_smem;       // 1: the triangular-solve vector lives in shared memory
   int y_bytes;      // bytes reserved for it (multiple of 128)
   int slot_bytes;   // bytes of one ring slot = largest stream chunk (multiple of 16)
+  int ring_bytes;   // bytes after the solve vector: the ring's slots, or tasks and the iteration's vector
   int dsm_bytes;    // total dynamic shared memory (ILUTP scratch may use all of it)
   int ilu64;        // 1: the ILUTP working row is FP64 whatever the stored precision
   int af_lag;       // background refactorisation: accepts between a snapshot and its use (0: off)
@@ -247,10 +248,13 @@ __device__ __forceinline__ int block_rows(const Walker& w, const Params& P) {
 constexpr int kLaneEntries = 8;  // entries of a lane in one task of a warp
 // Bytes of a task: words, sources, values.
 __host__ __device__ __forceinline__ constexpr int task_bytes(int tsz) { return 128 + 512 + 32 * kLaneEntries * tsz; }
-// Tasks of every warp that the shared memory after the solve area holds.
+// Tasks of every warp that the shared memory after the solve area holds (all of it: counted in
+// ring slots of 8 or 16 KB, FP64 walkers of n = 3456 and 4096 that share an SM missed the two
+// tasks a warp that they have room for, and solved level by level from chunk streams: 256 walkers
+// of n = 4096 434 us an apply of L and U, 190 from two tasks a warp; 160 of n = 3456 708 and 216).
 template <typename T>
 __device__ __forceinline__ int tasks_ahead(const Params& P) {
-  return P.ring_slots * P.slot_bytes / ((int)(blockDim.x >> 5) * task_bytes((int)sizeof(T)));
+  return P.ring_bytes / ((int)(blockDim.x >> 5) * task_bytes((int)sizeof(T)));
 }
 // Task streams serve the solves when the solve vector (and one block's intermediate one)
 // fit the shared-memory solve area, with 16-bit indices, blocks of a useful size and two

@@ -100,7 +100,7 @@ cudaError_t launch_bench_T(const LaunchCfg& L, const Walker* W, int nwalk, const
 // when they fit next to four ring slots and allow_sf (synchronisation-free triangular
 // solves), else one when it fits next to two slots, else none; then 16 KB slots when at
 // least four fit, else 8 KB.  Fills tri_sf, y_half, y_smem, y_bytes, ring_slots,
-// slot_bytes, dsm_bytes.
+// slot_bytes, ring_bytes, dsm_bytes.
 void plan_smem(int ybytes, int budget, Params& P, bool allow_sf);
 // Entries a row of the scratch of the blocked triangular solves (a multiple of 4).
 int expanded_row_cap(int capLU, int row_cap);

@@ -644,7 +644,7 @@ template <typename T>
 __device__ __forceinline__ T* z_ring(const Params& P) { return (T*)(dyn_smem() + P.y_bytes); }
 template <typename T>
 __device__ __forceinline__ bool krylov_in_smem(const Walker& w, const Params& P) {
-  return w.ctl->tri_tasks && (size_t)w.ld * sizeof(T) <= (size_t)P.ring_slots * P.slot_bytes;
+  return w.ctl->tri_tasks && (size_t)w.ld * sizeof(T) <= (size_t)P.ring_bytes;
 }
 template <typename T, bool SM>
 __device__ __forceinline__ void precond_apply(const Walker& w, const Params& P, const T* v, T* z, Shared& sh) {
