@@ -38,9 +38,9 @@ bool rows_fit_slot(int cap, int lfil_extra, int row_cap) {
 // streams are sized to match: a caller's cap stays the caller's.  n = 4096, fill limit that gave
 // blocks of 64 rows: 128 rows take the L and U solves of an iteration from 93 to 70 us, for
 // n x 64 more entries of scratch a factor set.
-static int block_scratch(int n, int capLU, int row_cap) {
+static int block_scratch(int n, int capLU, int row_cap, bool lean) {
   const int c = expanded_row_cap(capLU, row_cap);
-  return row_cap > 0 ? c : std::max(c, n >= 2048 ? kMaxBlk : 64);
+  return row_cap > 0 || lean ? c : std::max(c, n >= 2048 ? kMaxBlk : 64);
 }
 
 size_t stream_bytes(int n, int capLU, int exmax) {
@@ -157,6 +157,9 @@ struct vmc_ctx {
   cudaStream_t stream = nullptr;
   int threads = 256;
   int row_cap = 0;  // trisolve_row_cap
+  // the device had no room for the whole arena: without the transposed copies of the slots and
+  // the room for full blocks, which no result needs
+  bool lean = false;
   bool fp64 = false;
   std::vector<Walker> hw;
   Walker* dW = nullptr;
@@ -466,122 +469,127 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
   std::vector<size_t> ell_off(3 * (size_t)n_walkers);  // transposed slots: columns, FP64, FP32
   Carve cv;
   ctx->hw.resize(n_walkers);
-  long long base = 0;
-  for (int w = 0; w < n_walkers; ++w) {
-    const Layout& L = lay[w];
-    const int n = L.n, cap = L.cap, ld = pad4(n);
-    const int pmax = p.lfil_extra >= 0 ? p.lfil_extra : (cap + 1) / 2;
-    const int capLU = (cap + pmax + 2 + 3) / 4 * 4;  // rows of 16-byte multiples (bulk copies)
-    const int exb = block_scratch(n, capLU, p.trisolve_row_cap);
-    auto& o = offs[w];
-    o.push_back(cv.take<double>((size_t)n * 3));       // 0 Z
-    o.push_back(cv.take<int>(n));                      // 1 col_of_orb
-    o.push_back(cv.take<int>(n));                      // 2 orb_of_col
-    o.push_back(cv.take<double>((size_t)n * 3));       // 3 R
-    o.push_back(cv.take<int>(n));                      // 4 row_of_part
-    o.push_back(cv.take<int>(n));                      // 5 part_of_row
-    o.push_back(cv.take<int>((size_t)n * cap));        // 6 a_col
-    o.push_back(cv.take<double>((size_t)n * cap));     // 7 a_val
-    const bool ell = n < 0x10000;
-    o.push_back(cv.take<float>(ell ? 0 : (size_t)n * cap));  // 8 a_val32
-    o.push_back(cv.take<int>(n));                      // 9 a_len
-    o.push_back(cv.take<int>((size_t)n * capLU));      // 10 l_col
-    o.push_back(cv.take<double>((size_t)n * capLU));   // 11 l_val64
-    const size_t sbytes = stream_bytes(n, capLU, exb);
-    o.push_back(cv.take<unsigned char>(2 * sbytes));   // 12 lstream | ustream
-    o.push_back(cv.take<int>(n));                      // 13 l_len
-    o.push_back(cv.take<int>((size_t)n * capLU));      // 14 u_col
-    o.push_back(cv.take<double>((size_t)n * capLU));   // 15 u_val64
-    o.push_back(0);                                    // 16 (with 12)
-    o.push_back(cv.take<int>(n));                      // 17 u_len
-    o.push_back(cv.take<double>(n));                   // 18 u_dinv64
-    o.push_back(cv.take<int2>(2 * (size_t)n + 2));     // 19 lchunk | uchunk
-    o.push_back(cv.take<int>(n));                      // 20 perm
-    o.push_back(cv.take<int>(n));                      // 21 iperm
-    o.push_back(cv.take<int>(n));                      // 22 lev_l
-    o.push_back(cv.take<int>(n));                      // 23 lev_u
-    o.push_back(cv.take<int>(n + 1));                  // 24 l_lvl_ptr
-    o.push_back(cv.take<int>(n));                      // 25 l_lvl_rows
-    o.push_back(cv.take<int>(n + 1));                  // 26 u_lvl_ptr
-    o.push_back(cv.take<int>(n));                      // 27 u_lvl_rows
-    o.push_back(cv.take<int>(n + 1));                  // 28 lvl_cur
-    o.push_back(cv.take<double>(n));                   // 29 wrow
-    o.push_back(cv.take<int>(n));                      // 30 wpos
-    o.push_back(cv.take<int>(n));                      // 31 gP
-    o.push_back(cv.take<int>(n));                      // 32 gQ
-    o.push_back(cv.take<char>((size_t)mu * ld * Tsz)); // 33 upd_z
-    o.push_back(cv.take<int>((size_t)mu * kMaxU));     // 34 upd_ucol
-    o.push_back(cv.take<char>((size_t)mu * kMaxU * Tsz));  // 35 upd_uval
-    o.push_back(cv.take<int>(mu));                     // 36 upd_ulen
-    o.push_back(cv.take<double>((size_t)kMaxUpd * kMaxUpd));  // 37 upd_G
-    o.push_back(cv.take<char>((size_t)(m + 1) * ld * Tsz));   // 38 V
-    o.push_back(cv.take<char>((size_t)m * ld * Tsz));         // 39 Zk
-    o.push_back(cv.take<char>((size_t)3 * n * Tsz));          // 40 tv (three solve vectors)
-    o.push_back(cv.take<double>(n));                   // 41 x64
-    o.push_back(cv.take<double>(n));                   // 42 r64
-    o.push_back(cv.take<int>(cap));                    // 43 pend_acol
-    o.push_back(cv.take<double>(cap));                 // 44 pend_aval
-    o.push_back(cv.take<int>(kMaxU));                  // 45 pend_ucol
-    o.push_back(cv.take<double>(kMaxU));               // 46 pend_uval
-    o.push_back(cv.take<int4>(n + 1));                 // 47 chunk_meta
-    o.push_back(cv.take<int>(n + 1));                  // 48 lvl_nchunk
-    o.push_back(cv.take<int4>(2 * (size_t)n + 2));     // 49 seg_meta
-    if (ctx->pair) {
-      // second factor set (same order as offsets 10-30, 47-49), then the snapshot of A
-      o.push_back(cv.take<int>((size_t)n * capLU));    // 50 l_col
-      o.push_back(cv.take<double>((size_t)n * capLU)); // 51 l_val64
-      o.push_back(cv.take<unsigned char>(2 * sbytes)); // 52 lstream | ustream
-      o.push_back(cv.take<int>(n));                    // 53 l_len
-      o.push_back(cv.take<int>((size_t)n * capLU));    // 54 u_col
-      o.push_back(cv.take<double>((size_t)n * capLU)); // 55 u_val64
-      o.push_back(0);                                  // 56 (with 52)
-      o.push_back(cv.take<int>(n));                    // 57 u_len
-      o.push_back(cv.take<double>(n));                 // 58 u_dinv64
-      o.push_back(cv.take<int2>(2 * (size_t)n + 2));   // 59 lchunk | uchunk
-      o.push_back(cv.take<int>(n));                    // 60 perm
-      o.push_back(cv.take<int>(n));                    // 61 iperm
-      o.push_back(cv.take<int>(n));                    // 62 lev_l
-      o.push_back(cv.take<int>(n));                    // 63 lev_u
-      o.push_back(cv.take<int>(n + 1));                // 64 l_lvl_ptr
-      o.push_back(cv.take<int>(n));                    // 65 l_lvl_rows
-      o.push_back(cv.take<int>(n + 1));                // 66 u_lvl_ptr
-      o.push_back(cv.take<int>(n));                    // 67 u_lvl_rows
-      o.push_back(cv.take<int>(n + 1));                // 68 lvl_cur
-      o.push_back(cv.take<double>(n));                 // 69 wrow
-      o.push_back(cv.take<int>(n));                    // 70 wpos
-      o.push_back(cv.take<int4>(n + 1));               // 71 chunk_meta
-      o.push_back(cv.take<int>(n + 1));                // 72 lvl_nchunk
-      o.push_back(cv.take<int4>(2 * (size_t)n + 2));   // 73 seg_meta
-      o.push_back(cv.take<int>(n));                    // 74 snap_len
-      o.push_back(cv.take<int>((size_t)n * cap));      // 75 snap_col
-      o.push_back(cv.take<double>((size_t)n * cap));   // 76 snap_val
-      o.push_back(cv.take<int>(n));                    // 77 snap_part
-      o.push_back(cv.take<double>((size_t)n * 3));     // 78 snap_R
-      o.push_back(cv.take<int>(n));                    // 79 snap_rop
-      o.push_back(cv.take<int>(n));                    // 80 gP of the factor CTA
-      o.push_back(cv.take<int>(n));                    // 81 gQ of the factor CTA
+  auto carve_walkers = [&] {
+    cv = Carve();
+    long long base = 0;
+    for (int w = 0; w < n_walkers; ++w) {
+      const Layout& L = lay[w];
+      const int n = L.n, cap = L.cap, ld = pad4(n);
+      const int pmax = p.lfil_extra >= 0 ? p.lfil_extra : (cap + 1) / 2;
+      const int capLU = (cap + pmax + 2 + 3) / 4 * 4;  // rows of 16-byte multiples (bulk copies)
+      const int exb = block_scratch(n, capLU, p.trisolve_row_cap, ctx->lean);
+      auto& o = offs[w];
+      o.clear();
+      o.push_back(cv.take<double>((size_t)n * 3));       // 0 Z
+      o.push_back(cv.take<int>(n));                      // 1 col_of_orb
+      o.push_back(cv.take<int>(n));                      // 2 orb_of_col
+      o.push_back(cv.take<double>((size_t)n * 3));       // 3 R
+      o.push_back(cv.take<int>(n));                      // 4 row_of_part
+      o.push_back(cv.take<int>(n));                      // 5 part_of_row
+      o.push_back(cv.take<int>((size_t)n * cap));        // 6 a_col
+      o.push_back(cv.take<double>((size_t)n * cap));     // 7 a_val
+      const bool ell = n < 0x10000 && !ctx->lean;
+      o.push_back(cv.take<float>(ell ? 0 : (size_t)n * cap));  // 8 a_val32
+      o.push_back(cv.take<int>(n));                      // 9 a_len
+      o.push_back(cv.take<int>((size_t)n * capLU));      // 10 l_col
+      o.push_back(cv.take<double>((size_t)n * capLU));   // 11 l_val64
+      const size_t sbytes = stream_bytes(n, capLU, exb);
+      o.push_back(cv.take<unsigned char>(2 * sbytes));   // 12 lstream | ustream
+      o.push_back(cv.take<int>(n));                      // 13 l_len
+      o.push_back(cv.take<int>((size_t)n * capLU));      // 14 u_col
+      o.push_back(cv.take<double>((size_t)n * capLU));   // 15 u_val64
+      o.push_back(0);                                    // 16 (with 12)
+      o.push_back(cv.take<int>(n));                      // 17 u_len
+      o.push_back(cv.take<double>(n));                   // 18 u_dinv64
+      o.push_back(cv.take<int2>(2 * (size_t)n + 2));     // 19 lchunk | uchunk
+      o.push_back(cv.take<int>(n));                      // 20 perm
+      o.push_back(cv.take<int>(n));                      // 21 iperm
+      o.push_back(cv.take<int>(n));                      // 22 lev_l
+      o.push_back(cv.take<int>(n));                      // 23 lev_u
+      o.push_back(cv.take<int>(n + 1));                  // 24 l_lvl_ptr
+      o.push_back(cv.take<int>(n));                      // 25 l_lvl_rows
+      o.push_back(cv.take<int>(n + 1));                  // 26 u_lvl_ptr
+      o.push_back(cv.take<int>(n));                      // 27 u_lvl_rows
+      o.push_back(cv.take<int>(n + 1));                  // 28 lvl_cur
+      o.push_back(cv.take<double>(n));                   // 29 wrow
+      o.push_back(cv.take<int>(n));                      // 30 wpos
+      o.push_back(cv.take<int>(n));                      // 31 gP
+      o.push_back(cv.take<int>(n));                      // 32 gQ
+      o.push_back(cv.take<char>((size_t)mu * ld * Tsz)); // 33 upd_z
+      o.push_back(cv.take<int>((size_t)mu * kMaxU));     // 34 upd_ucol
+      o.push_back(cv.take<char>((size_t)mu * kMaxU * Tsz));  // 35 upd_uval
+      o.push_back(cv.take<int>(mu));                     // 36 upd_ulen
+      o.push_back(cv.take<double>((size_t)kMaxUpd * kMaxUpd));  // 37 upd_G
+      o.push_back(cv.take<char>((size_t)(m + 1) * ld * Tsz));   // 38 V
+      o.push_back(cv.take<char>((size_t)m * ld * Tsz));         // 39 Zk
+      o.push_back(cv.take<char>((size_t)3 * n * Tsz));          // 40 tv (three solve vectors)
+      o.push_back(cv.take<double>(n));                   // 41 x64
+      o.push_back(cv.take<double>(n));                   // 42 r64
+      o.push_back(cv.take<int>(cap));                    // 43 pend_acol
+      o.push_back(cv.take<double>(cap));                 // 44 pend_aval
+      o.push_back(cv.take<int>(kMaxU));                  // 45 pend_ucol
+      o.push_back(cv.take<double>(kMaxU));               // 46 pend_uval
+      o.push_back(cv.take<int4>(n + 1));                 // 47 chunk_meta
+      o.push_back(cv.take<int>(n + 1));                  // 48 lvl_nchunk
+      o.push_back(cv.take<int4>(2 * (size_t)n + 2));     // 49 seg_meta
+      if (ctx->pair) {
+        // second factor set (same order as offsets 10-30, 47-49), then the snapshot of A
+        o.push_back(cv.take<int>((size_t)n * capLU));    // 50 l_col
+        o.push_back(cv.take<double>((size_t)n * capLU)); // 51 l_val64
+        o.push_back(cv.take<unsigned char>(2 * sbytes)); // 52 lstream | ustream
+        o.push_back(cv.take<int>(n));                    // 53 l_len
+        o.push_back(cv.take<int>((size_t)n * capLU));    // 54 u_col
+        o.push_back(cv.take<double>((size_t)n * capLU)); // 55 u_val64
+        o.push_back(0);                                  // 56 (with 52)
+        o.push_back(cv.take<int>(n));                    // 57 u_len
+        o.push_back(cv.take<double>(n));                 // 58 u_dinv64
+        o.push_back(cv.take<int2>(2 * (size_t)n + 2));   // 59 lchunk | uchunk
+        o.push_back(cv.take<int>(n));                    // 60 perm
+        o.push_back(cv.take<int>(n));                    // 61 iperm
+        o.push_back(cv.take<int>(n));                    // 62 lev_l
+        o.push_back(cv.take<int>(n));                    // 63 lev_u
+        o.push_back(cv.take<int>(n + 1));                // 64 l_lvl_ptr
+        o.push_back(cv.take<int>(n));                    // 65 l_lvl_rows
+        o.push_back(cv.take<int>(n + 1));                // 66 u_lvl_ptr
+        o.push_back(cv.take<int>(n));                    // 67 u_lvl_rows
+        o.push_back(cv.take<int>(n + 1));                // 68 lvl_cur
+        o.push_back(cv.take<double>(n));                 // 69 wrow
+        o.push_back(cv.take<int>(n));                    // 70 wpos
+        o.push_back(cv.take<int4>(n + 1));               // 71 chunk_meta
+        o.push_back(cv.take<int>(n + 1));                // 72 lvl_nchunk
+        o.push_back(cv.take<int4>(2 * (size_t)n + 2));   // 73 seg_meta
+        o.push_back(cv.take<int>(n));                    // 74 snap_len
+        o.push_back(cv.take<int>((size_t)n * cap));      // 75 snap_col
+        o.push_back(cv.take<double>((size_t)n * cap));   // 76 snap_val
+        o.push_back(cv.take<int>(n));                    // 77 snap_part
+        o.push_back(cv.take<double>((size_t)n * 3));     // 78 snap_R
+        o.push_back(cv.take<int>(n));                    // 79 snap_rop
+        o.push_back(cv.take<int>(n));                    // 80 gP of the factor CTA
+        o.push_back(cv.take<int>(n));                    // 81 gQ of the factor CTA
+      }
+      o.push_back(cv.take<double2>(n));                  // u_head of factor set 0 (then of set 1)
+      if (ctx->pair) o.push_back(cv.take<double2>(n));
+      for (int sset = 0; sset < (ctx->pair ? 2 : 1); ++sset) {  // inverses of the diagonal blocks of each factor set
+        o.push_back(cv.take<int>(n));                      // ex_len
+        o.push_back(cv.take<int>((size_t)n * exb));        // ex_col
+        o.push_back(cv.take<double>((size_t)n * exb));     // ex_val
+      }
+      ell_off[w] = cv.take<unsigned short>(ell ? (size_t)cap * ld : 0);
+      ell_off[n_walkers + w] = cv.take<double>(ell ? (size_t)cap * ld : 0);
+      ell_off[2 * (size_t)n_walkers + w] = cv.take<float>(ell && !ctx->fp64 ? (size_t)cap * ld : 0);
+      Walker& W = ctx->hw[w];
+      std::memset(&W, 0, sizeof(W));
+      W.n = n; W.K = systems[w].K; W.lattice = systems[w].lattice; W.cap = cap; W.capLU = capLU;
+      W.m = m; W.mu = mu; W.ld = ld; W.per = L.per;
+      W.a = systems[w].a; W.kappa = systems[w].kappa; W.rc = systems[w].r_c;
+      W.rc2 = systems[w].r_c * systems[w].r_c; W.L = systems[w].K * systems[w].a;
+      W.log_base = base;
+      base += n;
+      ctx->max_n = std::max(ctx->max_n, n);
     }
-    o.push_back(cv.take<double2>(n));                  // u_head of factor set 0 (then of set 1)
-    if (ctx->pair) o.push_back(cv.take<double2>(n));
-    for (int sset = 0; sset < (ctx->pair ? 2 : 1); ++sset) {  // inverses of the diagonal blocks of each factor set
-      o.push_back(cv.take<int>(n));                      // ex_len
-      o.push_back(cv.take<int>((size_t)n * exb));        // ex_col
-      o.push_back(cv.take<double>((size_t)n * exb));     // ex_val
-    }
-    ell_off[w] = cv.take<unsigned short>(ell ? (size_t)cap * ld : 0);
-    ell_off[n_walkers + w] = cv.take<double>(ell ? (size_t)cap * ld : 0);
-    ell_off[2 * (size_t)n_walkers + w] = cv.take<float>(ell && !ctx->fp64 ? (size_t)cap * ld : 0);
-    Walker& W = ctx->hw[w];
-    std::memset(&W, 0, sizeof(W));
-    W.n = n; W.K = systems[w].K; W.lattice = systems[w].lattice; W.cap = cap; W.capLU = capLU;
-    W.m = m; W.mu = mu; W.ld = ld; W.per = L.per;
-    W.a = systems[w].a; W.kappa = systems[w].kappa; W.rc = systems[w].r_c;
-    W.rc2 = systems[w].r_c * systems[w].r_c; W.L = systems[w].K * systems[w].a;
-    W.log_base = base;
-    base += n;
-    ctx->max_n = std::max(ctx->max_n, n);
-  }
-  ctx->total_n = base;
+    ctx->total_n = base;
+  };
+  carve_walkers();
   {
     // shared-memory plan: the triangular-solve vector in shared memory when it fits,
     // and a ring of 2..8 chunk slots; aim for 2 CTAs per SM when walkers outnumber SMs
@@ -611,15 +619,25 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     ctx->smem = (size_t)ctx->P.dsm_bytes;
     ctx->smem_full = (size_t)budget1;
   }
-  const size_t ctl_off = cv.take<Ctl>(n_walkers);
-  const size_t walk_off = cv.take<Walker>(n_walkers);
-  const size_t energy_off = cv.take<double>(n_walkers);
-  const size_t budget_off = cv.take<unsigned long long>(1);
-  const size_t shadow_off = ctx->pair ? cv.take<Ctl>(n_walkers) : 0;
-  const size_t walk1_off = ctx->pair ? cv.take<Walker>(n_walkers) : 0;
-  const size_t walkf_off = ctx->pair ? cv.take<Walker>(2 * (size_t)n_walkers) : 0;
-  ctx->arena_bytes = cv.off + 256;
-  cudaError_t e = cudaMalloc((void**)&ctx->arena, ctx->arena_bytes);
+  size_t ctl_off = 0, walk_off = 0, energy_off = 0, budget_off = 0, shadow_off = 0, walk1_off = 0, walkf_off = 0;
+  auto allocate = [&] {
+    ctl_off = cv.take<Ctl>(n_walkers);
+    walk_off = cv.take<Walker>(n_walkers);
+    energy_off = cv.take<double>(n_walkers);
+    budget_off = cv.take<unsigned long long>(1);
+    shadow_off = ctx->pair ? cv.take<Ctl>(n_walkers) : 0;
+    walk1_off = ctx->pair ? cv.take<Walker>(n_walkers) : 0;
+    walkf_off = ctx->pair ? cv.take<Walker>(2 * (size_t)n_walkers) : 0;
+    ctx->arena_bytes = cv.off + 256;
+    return cudaMalloc((void**)&ctx->arena, ctx->arena_bytes);
+  };
+  cudaError_t e = allocate();
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    ctx->lean = true;
+    carve_walkers();
+    e = allocate();
+  }
   if (e != cudaSuccess) { *out = ctx; return cuda_fail(ctx, e, "cudaMalloc arena"); }
   e = cudaMemsetAsync(ctx->arena, 0, ctx->arena_bytes, ctx->stream);
   if (e != cudaSuccess) { *out = ctx; return cuda_fail(ctx, e, "cudaMemset arena"); }
@@ -639,7 +657,7 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     W.part_of_row = (int*)(A + o[5]);
     W.a_col = (int*)(A + o[6]);
     W.a_val = (double*)(A + o[7]);
-    if (W.n < 0x10000) {
+    if (W.n < 0x10000 && !ctx->lean) {
       W.ell_col = (unsigned short*)(A + ell_off[w]);
       W.ell_val = (double*)(A + ell_off[n_walkers + w]);
       if (!ctx->fp64) W.ell_val32 = (float*)(A + ell_off[2 * (size_t)n_walkers + w]);
@@ -653,7 +671,7 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     W.l_len = (int*)(A + o[13]);
     W.u_col = (int*)(A + o[14]);
     W.u_val64 = (double*)(A + o[15]);
-    W.sbytes = stream_bytes(W.n, W.capLU, block_scratch(W.n, W.capLU, ctx->row_cap));
+    W.sbytes = stream_bytes(W.n, W.capLU, block_scratch(W.n, W.capLU, ctx->row_cap, ctx->lean));
     W.ustream = W.lstream + W.sbytes;
     W.u_len = (int*)(A + o[17]);
     W.u_dinv64 = (double*)(A + o[18]);
@@ -692,7 +710,7 @@ extern "C" vmc_status vmc_create(const vmc_system* systems, int n_walkers, const
     W.u_head = (double2*)(A + o[ctx->pair ? 82 : 50]);
     {
       const size_t e0 = ctx->pair ? 84 : 51;
-      W.exmax = block_scratch(W.n, W.capLU, ctx->row_cap);
+      W.exmax = block_scratch(W.n, W.capLU, ctx->row_cap, ctx->lean);
       W.ex_len = (int*)(A + o[e0]);
       W.ex_col = (int*)(A + o[e0 + 1]);
       W.ex_val = (double*)(A + o[e0 + 2]);
