@@ -107,9 +107,9 @@ typedef struct {
                           to max_updates / 2; -1: auto -- on with max_updates / 2 when every
                           walker pair fits on the GPU at once (2 x walkers <= SMs) and no
                           system exceeds n = 8192 (beyond that one factorisation outlasts
-                          the accepts between adoptions and in-line refactoring is faster;
-                          at n = 32768 it takes about 28 s, near the 30 s bound on the
-                          solver's wait, past which the walker reports VMC_ERR_TIMEOUT) (-1) */
+                          the accepts between adoptions several times over; at n = 32768 it
+                          takes 3 to 15 s of the 30 s bound on the solver's wait, past which
+                          the walker reports VMC_ERR_TIMEOUT) (-1) */
   int refactor_reorder; /* background refactorisations first re-pair particles and orbitals
                           (the greedy reordering of Sec. 3.1) on the snapshot positions; the
                           solver adopts the new row order with the factors (0) */
@@ -153,8 +153,10 @@ typedef struct {
                           The same operator as row-by-row substitution in exact arithmetic.
                           0 or 1: level by level; ignored with trisolve = 1 (8) */
   int trisolve_row_cap; /* scratch of the blocked solves, entries a row, which bounds the rows of
-                          a block: 0 = max(c + 4, min(2 c, 160)) with c the factor-row capacity;
-                          otherwise max(c + 4, this), at most 480 (0) */
+                          a block: 0 = max(c + 4, min(2 c, 160)) with c the factor-row capacity,
+                          and in a context at least 64, from n = 2048 on 128, where device memory
+                          allows (vmc_ratio_noalloc: the first rule alone); otherwise
+                          max(c + 4, this), at most 480 (0) */
   int trisolve_lane_entries; /* triangular solves from the chunk streams (trisolve = 1,
                           trisolve_warp_rows > 0, or a solve vector that does not fit shared
                           memory): each row is summed by a group of lanes sized
@@ -403,7 +405,9 @@ vmc_status vmc_get_matrix(vmc_ctx* ctx, int walker, double* A_dense, int* part_o
  * (diagonal stored as 1), U upper, perm[t] = column of A_p in factor column t. */
 vmc_status vmc_get_factors(vmc_ctx* ctx, int walker, double* L_dense, double* U_dense, int* perm);
 /* Apply the current preconditioner M (Sec. 3.2 Eq. 18) of walker w to v (host, n,
- * indexed by rows of A_p) giving z (host, n, indexed by columns of A_p). */
+ * indexed by rows of A_p) giving z (host, n, indexed by columns of A_p).  In the working
+ * precision, by the solves in use: blocked ones multiply by inverses of diagonal blocks, which
+ * agree with substitution to a few roundings of the largest entry (1e-15 FP64, 4e-7 FP32). */
 vmc_status vmc_apply_preconditioner(vmc_ctx* ctx, int walker, const double* v, double* z);
 /* Force a reorder + refactorisation of walker w now (tests). */
 vmc_status vmc_refactor(vmc_ctx* ctx, int walker, int reorder);

@@ -238,10 +238,17 @@ struct __align__(16) Shared {
   double dflag[8];
 };
 
-// Blocked triangular solves (vmc_blocks.cuh): rows of a block.  From n = 2048 on the inverses
-// of 128-row blocks stay sparse (n = 4096, fill limit 32: 2.18 MB of streams against 2.23 MB
-// with 64 rows) and half the steps win: 80 against 98 us for L and U in FP32; below, the
-// larger blocks' inverses fill in (n = 343: 286 against 234 KB, 10.7 against 10.3 us).
+// Blocked triangular solves (vmc_blocks.cuh): rows of a block.  128 rows take half the steps;
+// their inverses hold more entries.  L and U of 64 walkers, us with 64 and with 128 rows in FP32
+// and in FP64, default fill limit (fill limit 32):
+//   n = 1000   15.3 13.0, 40.7 36.1  (21.8 20.9, 61.7 61.3; streams 568 717, 914 1158 KB)
+//   n = 1728   24.1 19.6, 66.1 54.6  (37.4 34.0, 106 96; 945 1111, 1521 1792 KB)
+//   n = 2197   31.6 25.8, 87.0 71.0  (48.4 42.2, 135 118; 1201 1372, 1934 2212 KB)
+//   n = 2744   38.3 30.9, 105 85.5   (58.9 50.9, 166 142)
+//   n = 4096   57.8 46.3, 156 125    (87.4 72.4, 248 201; 2242 2428, 3610 3915 KB)
+// and n = 343 10.3 10.7 in FP32 (234 286 KB).  From n = 2048 on they win by 13-20 % in both
+// precisions for 3-15 % more stream; the gain shrinks below, and the streams of many walkers
+// share the L2.  (The line could lie lower: n = 1728 gains 8-18 %.)
 __device__ __forceinline__ int block_rows(const Walker& w, const Params& P) {
   return min(min((w.n >= 2048 ? 16 : 8) * P.tri_group, kMaxBlk), w.exmax);
 }
@@ -427,10 +434,9 @@ __host__ __device__ __forceinline__ int chunk_bytes(int nseg, int r, int e, int 
   return kChunkHdr + 16 * nseg + 4 * pad4(r) + 4 * pad4(r + 1) + 4 * pad4(e) + pad16(tsz * e) +
          (upper ? pad16(tsz * r) : 0);
 }
-// Grouped form (header .w = 1): int4 seg[segments]; int4 rowdesc[r] {output index, first
-// entry, end entry, 0}; the entries: FP32 as (column bits, value) pairs of 8 bytes, FP64 as
-// an int column array then a double value array (12 bytes an entry: the streams of many
-// walkers share the L2).
+// Bytes of a chunk of rows with a 16-byte descriptor each and 8 (FP32) or 12 bytes an entry: no
+// stream has this form any more, but its longest row still bounds the parameters that vmc_create
+// accepts (rows_fit_slot).
 __host__ __device__ __forceinline__ int chunk_bytes_grouped(int nseg, int r, int e, int tsz) {
   return kChunkHdr + 16 * nseg + 16 * r + (tsz == 4 ? pad16(8 * e) : pad16(4 * e) + pad16(8 * e));
 }
