@@ -140,10 +140,11 @@ typedef struct {
                           hash map keyed by label when the dense working row of n entries does
                           not fit the shared memory (and n <= 65535), else the dense row; 1 =
                           always the dense row; 2 = always the hash map where it fits (0) */
-  int trisolve_warp_rows; /* level-by-level triangular solves from the chunk streams: a level of at most this many
-                          rows, <= 32, is solved by one warp alone, with no barrier among the
-                          solving warps after it (the other warps meet it before the next larger
-                          level); 0 = every level by all solving warps (0) */
+  int trisolve_warp_rows; /* level-by-level triangular solves (trisolve_group 0 or 1), then from the
+                          chunk streams: a level of at most this many rows, <= 32, is solved by one
+                          warp alone, with no barrier among the solving warps after it (the other
+                          warps meet it before the next larger level); 0 = every level by all
+                          solving warps; ignored by blocked solves (0) */
   int trisolve_group;  /* blocked triangular solves (a partitioned inverse of each factor): at
                           every factorisation the factor's rows are taken in blocks of 8 x this
                           many (16 x from n = 2048 on; at most 128, and at most the scratch of
@@ -158,7 +159,7 @@ typedef struct {
                           allows (vmc_ratio_noalloc: the first rule alone); otherwise
                           max(c + 4, this), at most 480 (0) */
   int trisolve_lane_entries; /* triangular solves from the chunk streams (trisolve = 1,
-                          trisolve_warp_rows > 0, or a solve vector that does not fit shared
+                          trisolve_warp_rows, or a solve vector that does not fit shared
                           memory): each row is summed by a group of lanes sized
                           for at most this many entries a lane on the level's
                           longest row, <= 64; 0 = 2 in FP32, 8 in FP64 (0) */

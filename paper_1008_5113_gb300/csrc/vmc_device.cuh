@@ -265,12 +265,12 @@ __device__ __forceinline__ int tasks_ahead(const Params& P) {
 }
 // Task streams serve the solves when the solve vector (and one block's intermediate one)
 // fit the shared-memory solve area, with 16-bit indices, blocks of a useful size and two
-// tasks a warp; else (and for the synchronisation-free solves and trisolve_warp_rows) the
-// level-ordered chunk streams.
+// tasks a warp; else (and for the synchronisation-free solves, and for trisolve_warp_rows where
+// the solves go level by level) the level-ordered chunk streams.
 template <typename T>
 __device__ __forceinline__ bool task_solves(const Walker& w, const Params& P) {
   const int B = P.tri_group > 1 ? block_rows(w, P) : 0;
-  return P.y_smem && !P.tri_sf && P.warp_rows == 0 && (P.tri_group <= 1 || (w.ex_col != nullptr && B >= 16)) &&
+  return P.y_smem && !P.tri_sf && (P.tri_group <= 1 ? P.warp_rows == 0 : w.ex_col != nullptr && B >= 16) &&
          w.n + B < 0xffff && (size_t)(w.n + B) * sizeof(T) <= (size_t)P.y_bytes && tasks_ahead<T>(P) >= 2;
 }
 

@@ -26,7 +26,7 @@ def vmc():
 
 @pytest.mark.parametrize("prec", [0, 1])
 @pytest.mark.parametrize("kw", [{}, dict(trisolve_group=1), dict(trisolve=1), dict(block_threads=64),
-                                dict(engine=1, trisolve_warp_rows=8)])
+                                dict(engine=1, trisolve_group=1, trisolve_warp_rows=8)])
 def test_lost_factorisation_is_reported(vmc, prec, kw):
     K, sigma = 6, 0.2
     s = O.system(K)

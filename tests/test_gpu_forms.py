@@ -57,6 +57,42 @@ def test_level_tasks_take_a_step_per_128_rows(vmc, prec, K, threads, kw):
         assert st["chunks_" + side] == int((-(-rows // 128)).sum())
 
 
+@pytest.mark.parametrize("prec", [0, 1])
+def test_warp_rows_leave_blocked_solves_alone(vmc, prec):
+    """trisolve_warp_rows is for level-by-level solves: with blocks the steps and the apply are
+    the same, bit for bit."""
+    s = O.system(7, 0, 1.0, 2.0, 1.45)
+    v = np.random.default_rng(3).standard_normal(343)
+    out = []
+    for rows in (0, 8, 32):
+        ctx = vmc.vmc_create([(7, 0, 1.0, 2.0, 1.45)], vmc.params(precision=prec, trisolve_warp_rows=rows))
+        try:
+            vmc.vmc_set_positions(ctx, 0, O.initial_positions(s, 5, 0.2))
+            st = vmc.vmc_get_stats(ctx, 0)
+            out.append((st["groups_L"], st["groups_U"], vmc.vmc_apply_preconditioner(ctx, 0, v).tobytes()))
+        finally:
+            vmc.vmc_destroy(ctx)
+    assert out[0][0] <= 12 and out[0] == out[1] == out[2]
+
+
+@pytest.mark.parametrize("K,threads", [(4, 0), (5, 64), (6, 96)])
+def test_dense_walkers_four_to_an_sm(vmc, K, threads):
+    """With more than two walkers an SM the dense kernels are compiled for four: the same walker's
+    log and positions, bit for bit."""
+    out = []
+    for walkers in (1, 310):
+        ctx = vmc.vmc_create([(K, 0, 1.0, 2.0, 1.5)] * walkers,
+                             vmc.params(precision=0, engine=vmc.ENGINE_DENSE_SM, block_threads=threads))
+        try:
+            vmc.vmc_init_positions(ctx, [5] * walkers, 0.1)
+            acc, rat = vmc.vmc_sweep(ctx, 2, 0.2, [7] * walkers)
+            out.append([(a.tobytes(), r.tobytes(), vmc.vmc_get_positions(ctx, w).tobytes())
+                        for w, (a, r) in enumerate(zip(acc.reshape(walkers, -1), rat.reshape(walkers, -1)))])
+        finally:
+            vmc.vmc_destroy(ctx)
+    assert all(x == out[0][0] for x in out[1])
+
+
 def test_flat_dense_form_gives_the_split_forms_logs(vmc):
     """A context with one walker too large for the split form takes the flat form for all of
     them.  That walker's matrix is singular (no particle near its first site), so it is given up
