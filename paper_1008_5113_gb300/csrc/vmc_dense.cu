@@ -162,6 +162,12 @@ __device__ __forceinline__ void cluster_sync(int size) {
     __syncthreads();
   }
 }
+// A load of what another CTA of the cluster may have written; a walker's only CTA reads its own
+// writes through L1.
+template <bool kSplit>
+__device__ __forceinline__ double ld_other(const double* p) {
+  return kSplit ? __ldcg(p) : *p;
+}
 struct DenseRows {
   int rank, size, lo, hi;  // this CTA's rows of B
 };
@@ -169,12 +175,21 @@ __device__ __forceinline__ DenseRows dense_rows(int n, int size) {
   const int rank = size > 1 ? cluster_rank() : 0;
   return DenseRows{rank, size, (int)((long long)n * rank / size), (int)((long long)n * (rank + 1) / size)};
 }
-constexpr int kBatch = 12;  // elements of a row a lane has in flight
+// Elements of a row that a lane has in flight: 12, or 4 in the kernels that are compiled for four
+// CTAs an SM (64 registers a thread).  Those serve walkers that would otherwise queue for an SM
+// (a sweep is a chain of short steps, which only other walkers fill) and rows of up to 128
+// elements, for which 12 batches of 32 are mostly loads past the row's end.  A sweep, ms, the
+// flat form before the split, 12 elements, 4: n = 64 x 250 walkers 1.58, 1.93, 1.54; x 600 3.16,
+// 3.80, 2.09; n = 125 x 250 4.82, 5.09, 3.93; n = 216 x 400 34.6, 23.3, 14.9.
+template <int kPerSm>
+constexpr int kBatchOf = kPerSm > 1 ? 4 : 12;
 // Shared memory of the split form: two rows, a column, the column permutation.
 __host__ __device__ __forceinline__ size_t dense_smem(int n) { return (size_t)n * (3 * 8 + 4); }
 
 // As dense_invert_flat, the CTA's rows of it.  Every CTA finds the pivot itself.
+template <int kPerSm, bool kSplit>
 __device__ __noinline__ bool dense_invert(const Walker& w, const DenseRows d, Shared& sh) {
+  constexpr int kBatch = kBatchOf<kPerSm>;
   const int n = w.n, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5, cap = w.cap;
   double* B = w.Bd;
   double* rk = (double*)dyn_smem();  // old row k
@@ -192,7 +207,7 @@ __device__ __noinline__ bool dense_invert(const Walker& w, const DenseRows d, Sh
     double bd = -1.0;
     int bi = k;
     for (int i = k + tid; i < n; i += nt) {
-      const double v = fabs(__ldcg(B + (size_t)i * n + k));
+      const double v = fabs(ld_other<kSplit>(B + (size_t)i * n + k));
       if (v > bd) { bd = v; bi = i; }
     }
     double neg = -bd;
@@ -201,8 +216,8 @@ __device__ __noinline__ bool dense_invert(const Walker& w, const DenseRows d, Sh
     if (-neg == 0.0) { ok = false; break; }
 #pragma unroll 4
     for (int j = tid; j < n; j += nt) {
-      rk[j] = __ldcg(B + (size_t)k * n + j);
-      rp[j] = __ldcg(B + (size_t)p * n + j);
+      rk[j] = ld_other<kSplit>(B + (size_t)k * n + j);
+      rp[j] = ld_other<kSplit>(B + (size_t)p * n + j);
     }
     if (tid == 0) piv[k] = p;
     __syncthreads();
@@ -270,8 +285,10 @@ __device__ __noinline__ bool dense_invert(const Walker& w, const DenseRows d, Sh
 
 // One Metropolis step of particle k, the CTA's rows of it; st: the walker's status, which
 // every CTA keeps alike.  The CTAs write the same matrix row and position.
+template <int kPerSm, bool kSplit>
 __device__ __forceinline__ void dense_step(const Walker& w, const DenseRows d, int k, uint64_t seed, uint32_t sweep,
                                            double sigma, uint8_t* acc_log, double* ratio_log, int& st, Shared& sh) {
+  constexpr int kBatch = kBatchOf<kPerSm>;
   const int n = w.n, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5, cap = w.cap;
   Ctl* c = w.ctl;
   if (tid == 0) {
@@ -294,7 +311,7 @@ __device__ __forceinline__ void dense_step(const Walker& w, const DenseRows d, i
   }
   double* B = w.Bd;
   double part = 0.0;
-  for (int t = tid; t < sh.ulen; t += nt) part += sh.uval[t] * __ldcg(B + (size_t)sh.ucol[t] * n + k);
+  for (int t = tid; t < sh.ulen; t += nt) part += sh.uval[t] * ld_other<kSplit>(B + (size_t)sh.ucol[t] * n + k);
   const double ratio = 1.0 + block_sum(part, sh);
   const double U = accept_uniform(seed, sweep, (uint32_t)k);
   const bool acc = __dmul_rn(ratio, ratio) > U;
@@ -313,7 +330,7 @@ __device__ __forceinline__ void dense_step(const Walker& w, const DenseRows d, i
   for (int b = tid; b < n; b += nt) {
     double s = 0.0;
 #pragma unroll 8
-    for (int t = 0; t < ulen; ++t) s = fma(sh.uval[t], __ldcg(B + (size_t)sh.ucol[t] * n + b), s);
+    for (int t = 0; t < ulen; ++t) s = fma(sh.uval[t], ld_other<kSplit>(B + (size_t)sh.ucol[t] * n + b), s);
     row[b] = s;
   }
   // every CTA has formed u from the old row and read the rows of u's support (a CTA may be
@@ -343,7 +360,8 @@ __device__ __forceinline__ void dense_step(const Walker& w, const DenseRows d, i
 }
 
 // split: rows over a cluster of `size` CTAs; else (size 0) one CTA in the flat form.
-__global__ void __launch_bounds__(kMaxThreads, 1) k_dense_setup(const Walker* __restrict__ W, int size) {
+template <int kPerSm, bool kSplit>
+__global__ void __launch_bounds__(kMaxThreads, kPerSm) k_dense_setup(const Walker* __restrict__ W, int size) {
   __shared__ Shared sh;
   const Walker& w = stage_walker(sh, W[blockIdx.x / max(size, 1)]);
   const DenseRows d = size ? dense_rows(w.n, size) : DenseRows{0, 1, 0, w.n};
@@ -357,7 +375,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_dense_setup(const Walker* __
     }
   }
   bad = __syncthreads_or(bad);
-  const bool ok = size ? dense_invert(w, d, sh) : dense_invert_flat(w, sh);
+  const bool ok = size ? dense_invert<kPerSm, kSplit>(w, d, sh) : dense_invert_flat(w, sh);
   if (threadIdx.x == 0 && d.rank == 0) {
     if (bad) w.ctl->status = ST_CAPACITY;
     else if (!ok) w.ctl->status = ST_BREAKDOWN;
@@ -365,7 +383,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_dense_setup(const Walker* __
   }
 }
 
-__global__ void __launch_bounds__(kMaxThreads, 1) k_dense_sweep(const Walker* __restrict__ W, int n_sweeps,
+template <int kPerSm, bool kSplit>
+__global__ void __launch_bounds__(kMaxThreads, kPerSm) k_dense_sweep(const Walker* __restrict__ W, int n_sweeps,
                                                              long long sweep0, double sigma,
                                                              const uint64_t* __restrict__ seeds, uint8_t* acc_log,
                                                              double* ratio_log, int refresh, int size) {
@@ -379,7 +398,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_dense_sweep(const Walker* __
   cluster_sync(size);      // read by all before the first can write it
   for (int s = 0; s < n_sweeps; ++s) {
     if (refresh > 0 && s > 0 && (sweep0 + s) % refresh == 0) {
-      const bool ok = size ? dense_invert(w, d, sh) : dense_invert_flat(w, sh);
+      const bool ok = size ? dense_invert<kPerSm, kSplit>(w, d, sh) : dense_invert_flat(w, sh);
       if (!ok) st = ST_BREAKDOWN;
       if (threadIdx.x == 0 && d.rank == 0) {
         w.ctl->factorizations += 1;
@@ -400,7 +419,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_dense_sweep(const Walker* __
       }
       uint8_t* al = acc_log ? acc_log + idx : nullptr;
       double* rl = ratio_log ? ratio_log + idx : nullptr;
-      if (size) dense_step(w, d, k, seed, (uint32_t)(sweep0 + s), sigma, al, rl, st, sh);
+      if (size) dense_step<kPerSm, kSplit>(w, d, k, seed, (uint32_t)(sweep0 + s), sigma, al, rl, st, sh);
       else dense_step_flat(w, k, seed, (uint32_t)(sweep0 + s), sigma, al, rl, sh);
       __syncthreads();
     }
@@ -419,12 +438,20 @@ static int dense_cluster(int nwalk, int max_n, int static_smem) {
   while (cs < 8 && 2 * cs * nwalk <= nsm) cs *= 2;
   return cs;
 }
+// kernels: for long rows and for many walkers or short rows (kBatchOf), each with rows split over
+// a cluster and with one CTA a walker.
 template <typename K, typename... A>
-static cudaError_t dense_launch(K kernel, const LaunchCfg& L, int nwalk, int max_n, A... args) {
+static cudaError_t dense_launch(const K (&kernels)[4], const LaunchCfg& L, int nwalk, int max_n, A... args) {
+  int dev = 0, nsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaFuncAttributes fa{};
-  const cudaError_t e = allow_dynamic_smem(kernel, &fa);
+  cudaError_t e = cudaFuncGetAttributes(&fa, kernels[0]);
   if (e != cudaSuccess) return e;
   const int cs = dense_cluster(nwalk, max_n, (int)fa.sharedSizeBytes);
+  const K kernel = kernels[2 * (nwalk > 2 * nsm || max_n <= 128) + (cs <= 1)];
+  e = allow_dynamic_smem(kernel);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3(std::max(cs, 1) * nwalk);
   lc.blockDim = dim3(L.threads);
@@ -441,11 +468,15 @@ static cudaError_t dense_launch(K kernel, const LaunchCfg& L, int nwalk, int max
 }
 
 cudaError_t launch_dense_setup(const LaunchCfg& L, const Walker* W, int nwalk, int max_n) {
-  return dense_launch(k_dense_setup, L, nwalk, max_n, W);
+  static constexpr decltype(&k_dense_setup<1, true>) kernels[] = {k_dense_setup<1, true>, k_dense_setup<1, false>,
+                                                                  k_dense_setup<4, true>, k_dense_setup<4, false>};
+  return dense_launch(kernels, L, nwalk, max_n, W);
 }
 cudaError_t launch_dense_sweep(const LaunchCfg& L, const Walker* W, int nwalk, int max_n, int n_sweeps, long long sweep0,
                                double sigma, const uint64_t* seeds, uint8_t* acc, double* ratio, int refresh) {
-  return dense_launch(k_dense_sweep, L, nwalk, max_n, W, n_sweeps, sweep0, sigma, seeds, acc, ratio, refresh);
+  static constexpr decltype(&k_dense_sweep<1, true>) kernels[] = {k_dense_sweep<1, true>, k_dense_sweep<1, false>,
+                                                                  k_dense_sweep<4, true>, k_dense_sweep<4, false>};
+  return dense_launch(kernels, L, nwalk, max_n, W, n_sweeps, sweep0, sigma, seeds, acc, ratio, refresh);
 }
 
 }  // namespace vmc

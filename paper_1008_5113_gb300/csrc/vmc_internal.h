@@ -22,13 +22,12 @@ struct LaunchCfg {
 // threads, and a context's own size, set before its launch, could be lowered by another's in
 // between ("too many resources requested for launch").  About 1 us of host time.
 template <typename K>
-cudaError_t allow_dynamic_smem(K kernel, cudaFuncAttributes* attributes = nullptr) {
+cudaError_t allow_dynamic_smem(K kernel) {
   cudaFuncAttributes fa{};
   int dev = 0, optin = 0;
   cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (attributes) *attributes = fa;
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
 }

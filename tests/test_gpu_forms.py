@@ -75,12 +75,12 @@ def test_warp_rows_leave_blocked_solves_alone(vmc, prec):
     assert out[0][0] <= 12 and out[0] == out[1] == out[2]
 
 
-@pytest.mark.parametrize("K,threads", [(4, 0), (5, 64), (6, 96)])
-def test_dense_walkers_four_to_an_sm(vmc, K, threads):
-    """With more than two walkers an SM the dense kernels are compiled for four: the same walker's
-    log and positions, bit for bit."""
+@pytest.mark.parametrize("K,threads", [(4, 0), (5, 64), (6, 96), (7, 0)])
+def test_dense_kernels_agree(vmc, K, threads):
+    """The dense kernels for rows split over a cluster and not, for long rows and for short rows or
+    more than two walkers an SM: the same walker's log and positions, bit for bit."""
     out = []
-    for walkers in (1, 310):
+    for walkers in (1, 160, 310):
         ctx = vmc.vmc_create([(K, 0, 1.0, 2.0, 1.5)] * walkers,
                              vmc.params(precision=0, engine=vmc.ENGINE_DENSE_SM, block_threads=threads))
         try:
@@ -90,7 +90,7 @@ def test_dense_walkers_four_to_an_sm(vmc, K, threads):
                         for w, (a, r) in enumerate(zip(acc.reshape(walkers, -1), rat.reshape(walkers, -1)))])
         finally:
             vmc.vmc_destroy(ctx)
-    assert all(x == out[0][0] for x in out[1])
+    assert all(x == out[0][0] for o in out for x in o)
 
 
 def test_flat_dense_form_gives_the_split_forms_logs(vmc):
